@@ -37,6 +37,7 @@
 
 #include "la.h"
 #include "la_device.cuh"
+#include "la_grid.cuh"
 
 using namespace la;
 
@@ -44,6 +45,16 @@ namespace {
 
 constexpr int kMaxDevices = 64;
 constexpr int kBlock = 256;
+
+// Control words of the end-of-phase kernel (k_sp_finish), beside Ctrl.
+struct FinCtrl {
+    GridBar bar;
+    int free_rows;                  // rows not yet matched in this phase (the refine counts down)
+    int count[2];                   // free rows listed in this round (double buffered)
+    int changed[3];                 // a potential fell in this sweep (triple buffered)
+    unsigned long long need[3];     // largest distance of a free row to a free column, per epoch
+    unsigned long long qmax[2];     // largest q before the update
+};
 
 __device__ __forceinline__ void sp_set_status(Ctrl *ctrl, int s) { atomicCAS(&ctrl->status, 0, s); }
 
@@ -99,7 +110,7 @@ __global__ void k_sp_qmin(const unsigned long long *__restrict__ key, int n, Ctr
 // shifted so that min q = 0, the price mirror refreshed, the queue reset.
 // zero = 1 restarts from zero prices (after the feasibility phase).
 __global__ void k_sp_reset(unsigned long long *__restrict__ key, unsigned long long *__restrict__ qm, int n,
-                           unsigned long long qlim, Ctrl *ctrl, int slot, int phase, int zero) {
+                           unsigned long long qlim, Ctrl *ctrl, FinCtrl *fin, int slot, int phase, int zero) {
     const unsigned long long qmin = zero ? 0ull : ctrl->qmin[slot];
     bool bad = false;
     for (int y = blockIdx.x * blockDim.x + threadIdx.x; y < n; y += gridDim.x * blockDim.x) {
@@ -113,7 +124,67 @@ __global__ void k_sp_reset(unsigned long long *__restrict__ key, unsigned long l
         ctrl->next_row = 0;
         ctrl->qmin[slot ^ 1] = ~0ull;
         ctrl->phase_start_scans[phase & 63] = ctrl->scans;
+        fin->free_rows = n;
+        for (int k = 0; k < 2; ++k) {
+            fin->count[k] = 0;
+            fin->qmax[k] = 0;
+        }
+        for (int k = 0; k < 3; ++k) {
+            fin->changed[k] = 0;
+            fin->need[k] = 0;
+        }
     }
+}
+
+// One bid of row `row` (a warp): best and second best of
+// v(x,y) = (C - cmin)(n+1) + q(y) over the row's arcs, then the double push
+// as one atomicMin on the column key. Returns the row left without a column
+// (the displaced one, `row` itself after a lost bid), or kMatched, or, with a
+// status set, kFailed.
+constexpr int kMatched = -1, kFailed = -2;
+template <bool ZERO>
+__device__ __forceinline__ int sp_bid(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ cols,
+                                      const int32_t *__restrict__ costs, int n, int cmin, uint32_t np1,
+                                      unsigned long long eps, unsigned long long qlim, unsigned long long qinf,
+                                      unsigned long long *__restrict__ key, unsigned long long *__restrict__ qm,
+                                      Ctrl *__restrict__ ctrl, int row, int lane, unsigned long long &wins,
+                                      unsigned long long &displaced) {
+    using V = unsigned long long;
+    const V inf = ~0ull;
+    const int b = __ldg(row_ptr + row), e = __ldg(row_ptr + row + 1);
+    ScanResult<V> r{inf, inf, 0, INT_MAX};
+    for (int k = b + lane; k < e; k += 32) {
+        const int y = __ldg(cols + k);
+        const V cs = ZERO ? 0ull : (V)(uint32_t)(__ldg(costs + k) - cmin) * np1;
+        const V v = cs + __ldcg(qm + y);
+        const bool better = v < r.b1 || (v == r.b1 && (unsigned)y < (unsigned)r.w);
+        const V hi = better ? r.b1 : v;
+        r.b2 = hi < r.b2 ? hi : r.b2;
+        r.c1 = better ? cs : r.c1;
+        r.w = better ? y : r.w;
+        r.b1 = better ? v : r.b1;
+    }
+    warp_merge(r);
+    if (r.b2 == inf) r.b2 = r.b1;     // a single arc: bid as on a tie
+    const unsigned long long nq = (r.b1 - r.c1) + (r.b2 - r.b1) + eps;
+    if (r.w >= n || nq > qlim || nq > qinf) {
+        if (lane == 0)
+            sp_set_status(ctrl, r.w >= n ? LA_ERR_INTERNAL : (nq > qinf ? LA_ERR_INFEASIBLE : LA_ERR_OVERFLOW));
+        return kFailed;
+    }
+    const unsigned long long nk = pack_key(nq, (uint32_t)row);
+    unsigned long long old = 0;
+    if (lane == 0) {
+        old = atomicMin(key + r.w, nk);
+        atomicMax(qm + r.w, old > nk ? nq : key_q(old));
+    }
+    old = __shfl_sync(0xffffffffu, old, 0);
+    if (old <= nk) return row;        // a lower price got there first: the row bids again
+    ++wins;
+    const uint32_t m = key_mate(old);
+    if (m == kNone) return kMatched;
+    ++displaced;
+    return (int)m;
 }
 
 // One refine phase over the arcs: persistent grid, one warp per free row.
@@ -124,16 +195,17 @@ __global__ void __launch_bounds__(kBlock)
 k_sp_refine(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ cols,
             const int32_t *__restrict__ costs, int n, int cmin, uint32_t np1, unsigned long long eps,
             unsigned long long qlim, unsigned long long qinf, unsigned long long *__restrict__ key,
-            unsigned long long *__restrict__ qm, Ctrl *__restrict__ ctrl, unsigned long long budget) {
+            unsigned long long *__restrict__ qm, Ctrl *__restrict__ ctrl, unsigned long long budget,
+            FinCtrl *__restrict__ fin, int hand_free) {
     constexpr unsigned kFlush = 8;
     const int lane = threadIdx.x & 31;
-    using V = unsigned long long;
-    const V inf = ~0ull;
     if (*reinterpret_cast<volatile int *>(&ctrl->status) != 0) return;   // an earlier phase failed
     int row = -1;
     unsigned long long wins = 0, displaced = 0, total = 0;
     unsigned pending = 0;
     for (;;) {
+        // few rows free: k_sp_finish ends the phase (the load overlaps the bid)
+        const int fr = __shfl_sync(0xffffffffu, *reinterpret_cast<volatile int *>(&fin->free_rows), 0);
         if (row < 0) {
             int r = 0;
             if (lane == 0) r = atomicAdd(&ctrl->next_row, 1);
@@ -158,45 +230,11 @@ k_sp_refine(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col
         }
         ++pending;
         ++total;
-        // best and second best of v(x,y) = (C - cmin)(n+1) + q(y) over the row's arcs
-        const int b = __ldg(row_ptr + row), e = __ldg(row_ptr + row + 1);
-        ScanResult<V> r{inf, inf, 0, INT_MAX};
-        for (int k = b + lane; k < e; k += 32) {
-            const int y = __ldg(cols + k);
-            const V cs = ZERO ? 0ull : (V)(uint32_t)(__ldg(costs + k) - cmin) * np1;
-            const V v = cs + __ldcg(qm + y);
-            const bool better = v < r.b1 || (v == r.b1 && (unsigned)y < (unsigned)r.w);
-            const V hi = better ? r.b1 : v;
-            r.b2 = hi < r.b2 ? hi : r.b2;
-            r.c1 = better ? cs : r.c1;
-            r.w = better ? y : r.w;
-            r.b1 = better ? v : r.b1;
-        }
-        warp_merge(r);
-        if (r.b2 == inf) r.b2 = r.b1;     // a single arc: bid as on a tie
-        const unsigned long long nq = (r.b1 - r.c1) + (r.b2 - r.b1) + eps;
-        if (r.w >= n || nq > qlim || nq > qinf) {
-            if (lane == 0)
-                sp_set_status(ctrl, r.w >= n ? LA_ERR_INTERNAL : (nq > qinf ? LA_ERR_INFEASIBLE : LA_ERR_OVERFLOW));
-            break;
-        }
-        const unsigned long long nk = pack_key(nq, (uint32_t)row);
-        unsigned long long old = 0;
-        if (lane == 0) {
-            old = atomicMin(key + r.w, nk);
-            atomicMax(qm + r.w, old > nk ? nq : key_q(old));
-        }
-        old = __shfl_sync(0xffffffffu, old, 0);
-        if (old > nk) {
-            ++wins;
-            const uint32_t m = key_mate(old);
-            if (m != kNone) {
-                ++displaced;
-                row = (int)m;
-            } else {
-                row = -1;
-            }
-        }
+        row = sp_bid<ZERO>(row_ptr, cols, costs, n, cmin, np1, eps, qlim, qinf, key, qm, ctrl, row, lane, wins,
+                           displaced);
+        if (row == kFailed) break;
+        if (row == kMatched && lane == 0) atomicSub(&fin->free_rows, 1);
+        if (fr <= hand_free) break;
     }
     if (lane == 0 && total) {
         atomicAdd(&ctrl->scans, (unsigned long long)pending);
@@ -204,6 +242,371 @@ k_sp_refine(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col
         atomicAdd(&ctrl->displaced, displaced);
         atomicAdd(&ctrl->full_scans, total);
         atomicMax(&ctrl->max_chain, total);
+    }
+}
+
+// The end of a phase: rounds of an exact global price update and of bids,
+// until no row is free. With few rows free the refine is one or a few serial
+// displacement chains of tens of thousands of bids (price wars: a column's
+// price rises by eps per bid); the update moves all those prices at once.
+//
+// The update (Sect. 5.2, Algorithm 5.3) with distances in price units
+// instead of buckets of eps: D(y) is the least length of a residual path
+// from column y to a free column, where the arc M(x) = y -> x -> z has
+// length l = v(x,z) - v(x,y) + eps >= 0 (eps-optimality). As a potential
+// S(y) = q(y) + D(y) it is the largest solution of
+//   S(y) = q(y) for a free column,
+//   S(y) <= min over the arcs x -> z, z != y, of c~(x,z) + S(z), + eps - c~(x,y)
+// found by Bellman-Ford sweeps that only ever lower S (values written by
+// other CTAs in the same sweep may be used). With q <- min(S, q + K) every
+// matched row stays eps-optimal: min(D(y), K) <= min(D(z), K) + l. K is the
+// largest distance of a free row, so that every free row's best arc then
+// starts a shortest path, and its bids walk along it (l = 0 up to ties)
+// unless the paths of two rows cross; such rows go into the next round. A
+// free row that reaches no free column has no augmenting path: no perfect
+// matching exists.
+//
+// Two bounds keep the sweeps short. The free rows' distances at the
+// potentials so far bound K from above: a column farther than that is not
+// lowered, and after two short epochs the arcs longer than that are dropped
+// (min(D, K) is the same). And the CTAs sweep on without waiting for each
+// other; grid barriers come once an epoch. A CTA keeps the arcs of its
+// columns' rows in shared memory for a round (8 bytes an arc, rows that find
+// no room are read from global memory), eight lanes per column (8..40 arcs a
+// row in the graphs this serves); only the potentials are gathered from L2.
+//
+// Measured on GB300, whole solves (mean of 6, ms), from one refine launch per
+// phase: sparse-uniform n = 65536, 33 arcs a row, 193 -> 29; sparse-geometric
+// n = 16384, 36 arcs a row, 242 -> 94. There the 50 updates take 58 ms (150
+// sweeps each, 4.5 us a sweep: gathers of 8 scattered bytes, about one 32-byte
+// sector per two cycles and SM), the bids 18 ms. Without the caching a sweep
+// took 19 us; without the bound on K 60 % more sweeps. Chains of at most 64,
+// 256 and 1024 bids a round: 107, 88 and 95 ms (and 36, 29, 31 on the uniform
+// graph): short chains do not reach the end of their path, long ones are rows
+// whose path was taken, in a price war that the next update ends sooner.
+constexpr int kFinBlock = 1024;
+constexpr int kFinLanes = 8;                                // lanes per column in a sweep
+constexpr int kFinPerWarp = 32 / kFinLanes;
+constexpr int kFinFirst = 6;                                // sweeps of a round's first epoch
+constexpr int kFinSweeps = 16;                              // sweeps of an epoch at most
+constexpr int kFinQuiet = 3;                                // ... and sweeps without a change that end it
+constexpr int kFinMinCols = 16;                             // columns per CTA at least
+constexpr int kFinMetaCap = 4096;                           // columns per CTA with cached arcs
+constexpr int kFinSmem = 200 * 1024;
+constexpr unsigned long long kFar = 1ull << 62;             // no path found yet
+constexpr int kFinBids = 256;                               // bids of a warp's chain in one round
+
+__device__ __forceinline__ unsigned long long min_u64_group(unsigned long long v) {
+#pragma unroll
+    for (int o = kFinLanes / 2; o; o >>= 1) {
+        const unsigned long long u = __shfl_xor_sync(0xffffffffu, v, o);
+        v = u < v ? u : v;
+    }
+    return v;
+}
+
+// *p read at L2 if `on`, else `other`; a predicated load, so that a lane's
+// loads are issued together whatever their predicates.
+__device__ __forceinline__ unsigned long long ld_if(const unsigned long long *p, bool on, unsigned long long other) {
+    unsigned long long v = other;
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\t@p ld.global.cg.u64 %0, [%1];\n\t}"
+                 : "+l"(v)
+                 : "l"(p), "r"((int)on)
+                 : "memory");
+    return v;
+}
+
+template <bool ZERO>
+__global__ void __launch_bounds__(kFinBlock)
+k_sp_finish(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ cols,
+            const int32_t *__restrict__ costs, int n, int cmin, uint32_t np1, unsigned long long eps,
+            unsigned long long qlim, unsigned long long qinf, unsigned long long *__restrict__ key,
+            unsigned long long *__restrict__ qm, unsigned long long *__restrict__ pot, int *__restrict__ rowcol,
+            int *__restrict__ rows, Ctrl *__restrict__ ctrl, unsigned long long budget, FinCtrl *__restrict__ fin,
+            int meta_cap, int arc_cap) {
+    extern __shared__ unsigned long long fin_smem[];
+    __shared__ int s_ok, s_used;
+    if (threadIdx.x == 0) s_ok = 1;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int gtid = blockIdx.x * blockDim.x + tid, gthreads = gridDim.x * blockDim.x;
+    const int sub = lane % kFinLanes;
+    // this CTA's columns: chunks of kFinMinCols (one 128-byte line of potentials), CTAs in turn
+    const int chunks = (n + kFinMinCols - 1) / kFinMinCols;
+    const int mine = kFinMinCols * ((chunks - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x);
+    auto column = [&](int j) {
+        return ((j / kFinMinCols) * (int)gridDim.x + (int)blockIdx.x) * kFinMinCols + j % kFinMinCols;
+    };
+    unsigned long long *s_cur = fin_smem;                                          // [meta_cap] S of the CTA's columns
+    unsigned long long *s_q = s_cur + meta_cap;                                    // [meta_cap] their prices
+    int2 *s_at = reinterpret_cast<int2 *>(s_q + meta_cap);                         // [meta_cap] first arc, padded count
+    unsigned *s_cy = reinterpret_cast<unsigned *>(s_at + meta_cap);                // [meta_cap] cost of the matched arc
+    int2 *s_arc = reinterpret_cast<int2 *>(s_cy + ((meta_cap + 1) & ~1));          // [arc_cap] column, cost - cmin
+    unsigned long long sweeps = 0;
+    unsigned long long wins = 0, displaced = 0, total = 0, longest = 0, updates = 0;
+    for (int round = 0;; ++round) {
+        const int par = round & 1;
+        // The status and the counters are read right after a barrier (or the
+        // launch), and are written again only after a further one: every CTA
+        // decides alike.
+        if (*reinterpret_cast<volatile int *>(&ctrl->status) != 0 ||
+            *reinterpret_cast<volatile int *>(&fin->free_rows) == 0)
+            break;
+        for (int x = gtid; x < n; x += gthreads) rowcol[x] = -1;
+        if (!grid_barrier(&fin->bar, &ctrl->status, &s_ok)) return;
+        unsigned long long qmx = 0;
+        for (int y = gtid; y < n; y += gthreads) {
+            const unsigned long long k = __ldcg(key + y);
+            const uint32_t x = key_mate(k);
+            qmx = max(qmx, key_q(k));
+            if (x < (uint32_t)n) {
+                rowcol[x] = y;
+                pot[y] = kFar;
+            } else {
+                pot[y] = key_q(k);
+            }
+        }
+        qmx = warp_max_u64(qmx);
+        if (lane == 0) atomicMax(&fin->qmax[par], qmx);
+        if (!grid_barrier(&fin->bar, &ctrl->status, &s_ok)) return;
+        for (int x = gtid; x < n; x += gthreads)
+            if (__ldcg(rowcol + x) < 0) rows[atomicAdd(&fin->count[par], 1)] = x;
+        // the arcs of this CTA's columns' rows into shared memory
+        if (tid == 0) s_used = 0;
+        __syncthreads();
+        for (int j0 = warp * kFinPerWarp; j0 < mine; j0 += (kFinBlock / 32) * kFinPerWarp) {
+            const int j = j0 + lane / kFinLanes;
+            int deg = 0, b = 0;
+            const int y = j < mine ? column(j) : n;
+            if (y < n) {
+                const uint32_t x = key_mate(__ldcg(key + y));
+                if (x < (uint32_t)n) {
+                    b = __ldg(row_ptr + x);
+                    deg = __ldg(row_ptr + x + 1) - b;
+                }
+            }
+            const int pad = (deg + kFinLanes - 1) / kFinLanes * kFinLanes;
+            int at = 0;
+            if (sub == 0 && pad) at = atomicAdd(&s_used, pad);
+            at = __shfl_sync(0xffffffffu, at, lane & ~(kFinLanes - 1));
+            const bool fits = at + pad <= arc_cap;
+            unsigned cy = 0xffffffffu;
+            for (int k = sub; k < pad; k += kFinLanes) {
+                int2 a = make_int2(-1, 0);     // no arc
+                if (k < deg) {
+                    a.x = __ldg(cols + b + k);
+                    a.y = ZERO ? 0 : __ldg(costs + b + k) - cmin;
+                    if (a.x == y) {    // the matched arc (the cheapest copy)
+                        cy = min(cy, (unsigned)a.y);
+                        a.x = -1;
+                    }
+                }
+                if (fits) s_arc[at + k] = a;
+            }
+#pragma unroll
+            for (int o = kFinLanes / 2; o; o >>= 1) cy = min(cy, __shfl_xor_sync(0xffffffffu, cy, o));
+            if (sub == 0 && y < n && j < meta_cap) {
+                s_cur[j] = deg ? kFar : 0ull;      // 0: a free column, nothing to lower
+                s_q[j] = key_q(__ldcg(key + y));
+                s_cy[j] = cy;
+                s_at[j] = fits ? make_int2(at, pad) : make_int2(-1, 0);
+            }
+        }
+        __syncthreads();
+        // Bellman-Ford sweeps until no potential falls. The CTAs sweep on
+        // without waiting for each other (S only falls, so any mix of old and
+        // new values is a valid relaxation) until kFinQuiet sweeps in a row
+        // changed nothing here; an epoch in which no CTA changed anything
+        // proves the fixed point.
+        unsigned long long lim = kFar;     // no column farther than this matters
+        for (int it = 0; it <= n + 1; ++it) {
+            const int slot = it % 3;
+            bool any = false;
+            if ((it == 2 || it == 4) && lim < kFar) {
+                // arcs longer than the limit cannot be on a path that matters:
+                // the cached rows keep the others
+                for (int j0 = warp * kFinPerWarp; j0 < mine; j0 += (kFinBlock / 32) * kFinPerWarp) {
+                    const int j = j0 + lane / kFinLanes;
+                    int2 at = make_int2(-1, 0);
+                    unsigned long long vm = 0;
+                    if (j < mine && column(j) < n && j < meta_cap && s_cur[j] != 0) {
+                        at = s_at[j];
+                        vm = (unsigned long long)s_cy[j] * np1 + s_q[j];
+                    }
+                    const int len = at.x >= 0 ? at.y : 0;
+                    const int longest_row = __reduce_max_sync(0xffffffffu, len);
+                    int w = 0;
+                    for (int k = sub; k < longest_row; k += kFinLanes) {   // longest_row: a multiple of kFinLanes
+                        int2 a = make_int2(-1, 0);
+                        bool keep = false;
+                        if (k < len) {
+                            a = s_arc[at.x + k];
+                            keep = a.x >= 0 &&
+                                   (unsigned long long)(unsigned)a.y * np1 + __ldcg(qm + a.x) + eps <= vm + lim;
+                        }
+                        const unsigned votes = __ballot_sync(0xffffffffu, keep) >> (lane & ~(kFinLanes - 1));
+                        if (keep) s_arc[at.x + w + __popc(votes & ((1u << sub) - 1))] = a;   // at or before its old place
+                        w += __popc(votes & ((1u << kFinLanes) - 1));
+                        __syncwarp();
+                    }
+                    const int pad = (w + kFinLanes - 1) / kFinLanes * kFinLanes;
+                    if (len && w + sub < pad) s_arc[at.x + w + sub] = make_int2(-1, 0);
+                    if (len && sub == 0) s_at[j].y = pad;
+                }
+                __syncthreads();
+            }
+            const int most = it < 2 ? kFinFirst : kFinSweeps;
+            for (int sw = 0, quiet = 0; sw < most && quiet < kFinQuiet; ++sw) {
+                bool fell = false;
+                for (int j0 = warp * kFinPerWarp; j0 < mine; j0 += (kFinBlock / 32) * kFinPerWarp) {
+                    const int j = j0 + lane / kFinLanes;
+                    const int y = j < mine ? column(j) : n;
+                    unsigned long long best = kFar, cur = 0, q = 0;
+                    unsigned cy = 0;
+                    if (y < n && j < meta_cap) {
+                        cur = s_cur[j];
+                        q = s_q[j];
+                        cy = s_cy[j];
+                        const int2 at = s_at[j];
+                        if (cur != 0 && at.x >= 0) {
+                            // four gathers in flight per lane
+                            for (int k = sub; k < at.y; k += 4 * kFinLanes) {
+                                unsigned long long v[4];
+                                unsigned c[4];
+#pragma unroll
+                                for (int g = 0; g < 4; ++g) {
+                                    int2 a = make_int2(-1, 0);
+                                    if (k + g * kFinLanes < at.y) a = s_arc[at.x + k + g * kFinLanes];
+                                    c[g] = (unsigned)a.y;
+                                    v[g] = ld_if(pot + max(a.x, 0), a.x >= 0, kFar);
+                                }
+#pragma unroll
+                                for (int g = 0; g < 4; ++g) best = min(best, (unsigned long long)c[g] * np1 + v[g]);
+                            }
+                        }
+                    }
+                    // a row that found no room: its arcs from global memory
+                    if (y < n && (j >= meta_cap || (cur != 0 && s_at[j].x < 0))) {
+                        const unsigned long long ky = __ldcg(key + y);
+                        const uint32_t x = key_mate(ky);
+                        q = key_q(ky);
+                        cur = x < (uint32_t)n ? __ldcg(pot + y) : 0ull;
+                        if (cur != 0) {
+                            const int b = __ldg(row_ptr + x), e = __ldg(row_ptr + x + 1);
+                            cy = 0xffffffffu;
+                            for (int k = b; k < e; ++k)
+                                if (!ZERO && __ldg(cols + k) == y) cy = min(cy, (unsigned)(__ldg(costs + k) - cmin));
+                            if (ZERO) cy = 0;
+                            for (int k = b + sub; k < e; k += kFinLanes) {
+                                const int z = __ldg(cols + k);
+                                if (z == y) continue;
+                                const unsigned c = ZERO ? 0u : (unsigned)(__ldg(costs + k) - cmin);
+                                best = min(best, (unsigned long long)c * np1 + __ldcg(pot + z));
+                            }
+                        }
+                    }
+                    best = min_u64_group(best);
+                    if (sub == 0 && best < kFar && best + eps < cur + (unsigned long long)cy * np1) {
+                        const unsigned long long v = best + eps - (unsigned long long)cy * np1;
+                        if (v <= q + lim) {
+                            __stcg(pot + y, v);
+                            if (j < meta_cap) s_cur[j] = v;
+                            fell = true;
+                        }
+                    }
+                }
+                ++sweeps;
+                const bool f = __syncthreads_or(fell) != 0;
+                any |= f;
+                quiet = f ? 0 : quiet + 1;
+            }
+            if (any && tid == 0) fin->changed[slot] = 1;
+            // The free rows' distances at the potentials so far bound the
+            // level K from above. (The list of free rows is complete from the
+            // second epoch on.)
+            unsigned long long far = 0;
+            if (it > 0) {
+                const int count = __ldcg(&fin->count[par]);
+                for (int i = warp * gridDim.x + blockIdx.x; i < count; i += gridDim.x * (blockDim.x >> 5)) {
+                    const int x = __ldcg(rows + i);
+                    const int b = __ldg(row_ptr + x), e = __ldg(row_ptr + x + 1);
+                    unsigned long long m = ~0ull, t = ~0ull;
+                    for (int k = b + lane; k < e; k += 32) {
+                        const int z = __ldg(cols + k);
+                        const unsigned long long c =
+                            ZERO ? 0ull : (unsigned long long)(uint32_t)(__ldg(costs + k) - cmin) * np1;
+                        m = min(m, c + __ldcg(qm + z));
+                        t = min(t, c + __ldcg(pot + z));
+                    }
+                    m = warp_min(m);
+                    t = warp_min(t);
+                    far = max(far, t >= kFar ? kFar : t - m);
+                }
+            }
+            if (lane == 0 && far) atomicMax(&fin->need[slot], far);
+            // the next epoch's words were last read before the barrier every CTA has passed since
+            if (gtid == 0) {
+                fin->changed[(it + 1) % 3] = 0;
+                fin->need[(it + 1) % 3] = 0;
+            }
+            if (!grid_barrier(&fin->bar, &ctrl->status, &s_ok)) return;
+            if (it == 0) continue;
+            lim = *reinterpret_cast<volatile unsigned long long *>(&fin->need[slot]);
+            if ( *reinterpret_cast<volatile int *>(&fin->changed[slot]) == 0) break;
+        }
+        ++updates;
+        // lim is now the largest distance of a free row: the level K
+        if (lim >= kFar && gtid == 0) sp_set_status(ctrl, LA_ERR_INFEASIBLE);
+        const int count = *reinterpret_cast<volatile int *>(&fin->count[par]);
+        if (!grid_barrier(&fin->bar, &ctrl->status, &s_ok)) return;
+        if (*reinterpret_cast<volatile int *>(&ctrl->status) != 0) break;
+        const unsigned long long qmax = *reinterpret_cast<volatile unsigned long long *>(&fin->qmax[par]);
+        const unsigned long long K = min(lim, qlim > qmax ? qlim - qmax : 0ull);
+        for (int y = gtid; y < n && K > 0; y += gthreads) {
+            const unsigned long long k = __ldcg(key + y);
+            const unsigned long long q = key_q(k), s = __ldcg(pot + y), nq = s < q + K ? max(s, q) : q + K;
+            if (nq == q) continue;
+            key[y] = pack_key(nq, key_mate(k));
+            qm[y] = nq;
+        }
+        if (gtid == 0) {   // the other parity's counters, for the next round
+            fin->count[par ^ 1] = 0;
+            fin->qmax[par ^ 1] = 0;
+            for (int k = 0; k < 3; ++k) {   // every sweep's words have been read
+                fin->changed[k] = 0;
+                fin->need[k] = 0;
+            }
+        }
+        if (!grid_barrier(&fin->bar, &ctrl->status, &s_ok)) return;
+        // the free rows bid, one warp per row, spread over the SMs first
+        for (int i = warp * gridDim.x + blockIdx.x; i < count; i += gridDim.x * (blockDim.x >> 5)) {
+            int row = __ldcg(rows + i);
+            unsigned steps = 0;
+            while (row >= 0 && steps < (unsigned)kFinBids) {
+                ++steps;
+                row = sp_bid<ZERO>(row_ptr, cols, costs, n, cmin, np1, eps, qlim, qinf, key, qm, ctrl, row, lane, wins,
+                                   displaced);
+            }
+            if (row == kMatched && lane == 0) atomicSub(&fin->free_rows, 1);
+            total += steps;
+            longest = max(longest, (unsigned long long)steps);
+            unsigned long long sc = 0;
+            if (lane == 0) {
+                sc = atomicAdd(&ctrl->scans, (unsigned long long)steps) + steps;
+                if (sc > budget) sp_set_status(ctrl, LA_ERR_ITER_LIMIT);
+            }
+            if (row == kFailed) break;
+        }
+        if (!grid_barrier(&fin->bar, &ctrl->status, &s_ok)) return;
+    }
+    if (lane == 0 && total) {
+        atomicAdd(&ctrl->wins, wins);
+        atomicAdd(&ctrl->displaced, displaced);
+        atomicAdd(&ctrl->full_scans, total);
+        atomicMax(&ctrl->max_chain, longest);
+    }
+    if (gtid == 0) {
+        ctrl->pu_updates += updates;
+        ctrl->pu_iters += sweeps;      // of the first CTA
     }
 }
 
@@ -243,6 +646,10 @@ struct SparseWorkspace {
     unsigned long long *key = nullptr;
     unsigned long long *qm = nullptr;
     int *colseen = nullptr;
+    unsigned long long *pot = nullptr;   // end-of-phase kernel: potentials, row -> column, free rows
+    int *rowcol = nullptr;
+    int *rows = nullptr;
+    FinCtrl *fin = nullptr;
     Ctrl *ctrl = nullptr;
     Ctrl *h_ctrl = nullptr;
     int num_sms = 0;
@@ -268,11 +675,18 @@ la_status ensure_sws(SparseWorkspace &w, int64_t n) {
         int o = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_sp_refine<false>, kBlock, 0);
         w.occ = std::max(1, o);
+        if (cudaMalloc(&w.fin, sizeof(FinCtrl)) != cudaSuccess) return LA_ERR_NOMEM;
     }
     if (w.cap < n) {
         cudaFree(w.key);
         cudaFree(w.qm);
         cudaFree(w.colseen);
+        cudaFree(w.pot);
+        cudaFree(w.rowcol);
+        cudaFree(w.rows);
+        w.pot = nullptr;
+        w.rowcol = nullptr;
+        w.rows = nullptr;
         w.key = nullptr;
         w.qm = nullptr;
         w.colseen = nullptr;
@@ -281,9 +695,41 @@ la_status ensure_sws(SparseWorkspace &w, int64_t n) {
         if (cudaMalloc(&w.key, sizeof(unsigned long long) * cap) != cudaSuccess) return LA_ERR_NOMEM;
         if (cudaMalloc(&w.qm, sizeof(unsigned long long) * cap) != cudaSuccess) return LA_ERR_NOMEM;
         if (cudaMalloc(&w.colseen, sizeof(int) * cap) != cudaSuccess) return LA_ERR_NOMEM;
+        if (cudaMalloc(&w.pot, sizeof(unsigned long long) * cap) != cudaSuccess) return LA_ERR_NOMEM;
+        if (cudaMalloc(&w.rowcol, sizeof(int) * cap) != cudaSuccess) return LA_ERR_NOMEM;
+        if (cudaMalloc(&w.rows, sizeof(int) * cap) != cudaSuccess) return LA_ERR_NOMEM;
         w.cap = cap;
     }
     return LA_OK;
+}
+
+// Free rows at which the refine hands a phase to the end-of-phase kernel.
+// Measured (means of 6 solves, ms) at n / 1000, n / 128, n / 32: sparse-uniform
+// n = 65536 73, 29, 28; sparse-geometric n = 16384 273, 88, 94.
+int sp_hand_free(int n) {
+    return std::max(8, n / 64);
+}
+
+// The end-of-phase kernel on a co-resident grid: one CTA per SM, fewer when
+// the graph has fewer columns than the grid has lane groups.
+template <bool ZERO>
+cudaError_t launch_finish(cudaStream_t s, SparseWorkspace &w, const int32_t *row_ptr, const int32_t *cols,
+                          const int32_t *costs, int n, int cmin, uint32_t np1, unsigned long long eps,
+                          unsigned long long qlim, unsigned long long qinf, unsigned long long budget) {
+    const int grid = std::max(1, std::min(w.num_sms, (n + kFinMinCols - 1) / kFinMinCols));
+    // shared memory: what this graph needs, up to kFinSmem
+    const int chunks = (n + kFinMinCols - 1) / kFinMinCols;
+    int meta_cap = std::min(kFinMetaCap, kFinMinCols * ((chunks + grid - 1) / grid));
+    const int meta = 24 * meta_cap + 4 * ((meta_cap + 1) & ~1);
+    int arc_cap = (kFinSmem - meta) / 8;
+    const cudaError_t e =
+        cudaFuncSetAttribute(k_sp_finish<ZERO>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFinSmem);
+    if (e != cudaSuccess) return e;
+    void *args[] = {(void *)&row_ptr, (void *)&cols, (void *)&costs, (void *)&n, (void *)&cmin, (void *)&np1,
+                    (void *)&eps, (void *)&qlim, (void *)&qinf, (void *)&w.key, (void *)&w.qm, (void *)&w.pot,
+                    (void *)&w.rowcol, (void *)&w.rows, (void *)&w.ctrl, (void *)&budget, (void *)&w.fin,
+                    (void *)&meta_cap, (void *)&arc_cap};
+    return cudaLaunchCooperativeKernel((const void *)k_sp_finish<ZERO>, dim3(grid), dim3(kFinBlock), args, kFinSmem, s);
 }
 
 }  // namespace
@@ -325,6 +771,7 @@ static la_status sparse_locked(const int32_t *row_ptr, const int32_t *cols, cons
     *w.h_ctrl = init;
     LA_SCK(cudaMemcpyAsync(w.ctrl, w.h_ctrl, sizeof(Ctrl), cudaMemcpyHostToDevice, s));
     LA_SCK(cudaMemsetAsync(w.colseen, 0, sizeof(int) * n, s));
+    LA_SCK(cudaMemsetAsync(w.fin, 0, sizeof(FinCtrl), s));
     int64_t launches = 0;
     const int vg = std::max(1, std::min((std::max(n, nnz) + kBlock - 1) / kBlock, 8 * w.num_sms));
     k_sp_validate<<<vg, kBlock, 0, s>>>(row_ptr, cols, costs, n, nnz, w.colseen, w.ctrl);
@@ -359,11 +806,14 @@ static la_status sparse_locked(const int32_t *row_ptr, const int32_t *cols, cons
                                                               : 256ull * n * (sched.size() + 1) + (1ull << 22);
     const int grid = std::max(1, std::min(w.num_sms * w.occ, (n + kBlock / 32 - 1) / (kBlock / 32)));
     if (profile) LA_SCK(cudaEventRecord(w.ev[0], s));
+    const int hand_free = sp_hand_free(n);
+    const unsigned long long qinf = 4ull * (unsigned long long)n + 4;
     // feasibility phase: zero costs, eps = 1, prices from 0
-    k_sp_reset<<<sg, kBlock, 0, s>>>(w.key, w.qm, n, qlim, w.ctrl, 0, 0, 1);
+    k_sp_reset<<<sg, kBlock, 0, s>>>(w.key, w.qm, n, qlim, w.ctrl, w.fin, 0, 0, 1);
     k_sp_refine<true><<<grid, kBlock, 0, s>>>(row_ptr, cols, costs, n, c0.cmin, (uint32_t)np1, 1ull, qlim,
-                                              4ull * (unsigned long long)n + 4, w.key, w.qm, w.ctrl, budget);
-    launches += 2;
+                                              qinf, w.key, w.qm, w.ctrl, budget, w.fin, hand_free);
+    LA_SCK(launch_finish<true>(s, w, row_ptr, cols, costs, n, c0.cmin, (uint32_t)np1, 1ull, qlim, qinf, budget));
+    launches += 3;
     // cost phases (Algorithm 5.0), from zero prices again
     int ph = 0;
     for (; ph < (int)sched.size(); ++ph) {
@@ -372,10 +822,12 @@ static la_status sparse_locked(const int32_t *row_ptr, const int32_t *cols, cons
             k_sp_qmin<<<sg, kBlock, 0, s>>>(w.key, n, w.ctrl, slot);
             ++launches;
         }
-        k_sp_reset<<<sg, kBlock, 0, s>>>(w.key, w.qm, n, qlim, w.ctrl, slot, ph + 1, ph == 0);
+        k_sp_reset<<<sg, kBlock, 0, s>>>(w.key, w.qm, n, qlim, w.ctrl, w.fin, slot, ph + 1, ph == 0);
         k_sp_refine<false><<<grid, kBlock, 0, s>>>(row_ptr, cols, costs, n, c0.cmin, (uint32_t)np1, sched[ph],
-                                                   qlim, ~0ull, w.key, w.qm, w.ctrl, budget);
-        launches += 2;
+                                                   qlim, ~0ull, w.key, w.qm, w.ctrl, budget, w.fin, hand_free);
+        LA_SCK(launch_finish<false>(s, w, row_ptr, cols, costs, n, c0.cmin, (uint32_t)np1, sched[ph], qlim, ~0ull,
+                                    budget));
+        launches += 3;
     }
     if (profile) LA_SCK(cudaEventRecord(w.ev[1], s));
     const int fslot = ph & 1;
@@ -397,7 +849,9 @@ static la_status sparse_locked(const int32_t *row_ptr, const int32_t *cols, cons
     stats.wins = (int64_t)c1.wins;
     stats.displaced = (int64_t)c1.displaced;
     stats.launches = launches;
-    stats.refine_launches = (int64_t)sched.size() + 1;
+    stats.refine_launches = 2 * ((int64_t)sched.size() + 1);
+    stats.price_updates = (int64_t)c1.pu_updates;
+    stats.price_update_sweeps = (int64_t)c1.pu_iters;
     stats.max_chain = (int64_t)c1.max_chain;
     stats.full_scans = (int64_t)c1.full_scans;
     for (int k = 0; k <= ph && k < LA_STATS_PHASES; ++k) {

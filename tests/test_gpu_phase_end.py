@@ -58,3 +58,24 @@ def test_no_augmenting_path_is_infeasible(la, n):  # noqa: F811
         arcs += [(x, x, 1), (x, x - 1, 2)]
     rp, cols, costs = to_csr(n, arcs)
     assert gpu_solve(la, rp, cols, costs).stats["status"] == la.LA_ERR_INFEASIBLE
+
+
+@pytest.mark.parametrize("n", [1, 2, 31, 33, 130, 513, 1026])
+def test_certificate_is_the_largest_potential(la, n):  # noqa: F811
+    """la_dual_certificate equals plain Bellman-Ford on the residual graph
+    (a unique fixed point), for widths with and without 16-byte rows."""
+    import torch
+    C = synth.geometric_costs(n, 3 + n)
+    t = torch.from_numpy(C).cuda()
+    match = la.solve(t).match
+    u, v = (a.cpu().numpy() for a in la.dual_certificate(t, match))
+    m = match.cpu().numpy()
+    c, on = C.astype(np.int64), C[np.arange(n), m].astype(np.int64)
+    want = np.zeros(n, np.int64)
+    for _ in range(n + 2):
+        new = np.minimum(want, (c + (want[m] - on)[:, None]).min(0))
+        if np.array_equal(new, want):
+            break
+        want = new
+    np.testing.assert_array_equal(v, want)
+    np.testing.assert_array_equal(u, on - want[m])

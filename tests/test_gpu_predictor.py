@@ -211,3 +211,26 @@ def test_trained_predictor_gains_over_cold_start(la):
         cold_scans += cold.stats["scans"]
         warm_scans += warm.stats["scans"]
     assert warm_scans < 0.6 * cold_scans, (warm_scans, cold_scans)
+
+
+@pytest.mark.parametrize("sizes", [[2], [63], [64], [65], [1, 127, 1], [128, 129], [700, 3, 1000]])
+def test_gradients_at_tile_edges(la, sizes):
+    """Rows around the 64-row tiles of the backward glue and the 128-row tiles
+    of the products, segments that straddle them, one and many K splits. The
+    oracle rounds the same operands to BF16, so the products differ by the
+    order of their FP32 sums only: the bound is test_gradients_match_oracle's."""
+    import torch
+    P = _params(13)
+    X, t, seg = _inputs(14, sizes)
+    g = torch.zeros(la.LA_PRED_PARAMS, dtype=torch.float32, device="cuda")
+    loss = ctypes.c_float(0)
+    rc = la.la_predictor_train_step(_dev(P, np.float32), None, None, _dev(X, np.float32), _dev(t, np.float32),
+                                    _dev(seg, np.int32), len(seg) - 1, X.shape[0], 1, 0.0, 0.0, None, g,
+                                    ctypes.byref(loss))
+    assert rc == la.LA_OK
+    Lq, gq = se.loss_grad(P.astype(np.float32).astype(np.float64), X, t, seg, quant=True)
+    assert loss.value == pytest.approx(Lq, rel=5e-3)
+    g = g.cpu().numpy().astype(np.float64)
+    for a, b in ((se.OFF_W1, se.OFF_B1), (se.OFF_B1, se.OFF_W2), (se.OFF_W2, se.OFF_B2), (se.OFF_B2, se.OFF_W3),
+                 (se.OFF_W3, se.OFF_B3)):
+        assert np.linalg.norm(g[a:b] - gq[a:b]) < 5e-3 * max(np.linalg.norm(gq[a:b]), 1e-12)

@@ -131,3 +131,18 @@ def test_round_limit_then_a_clean_solve(la):
     res = gpu_flow(la, *g, cycle=1, max_rounds=1)
     assert res.stats["status"] == la.LA_ERR_ITER_LIMIT
     expect_same(la, *g)
+
+
+@pytest.mark.parametrize("H,W", [(1, 1), (1, 70), (31, 33), (32, 32), (33, 64), (65, 97)])
+def test_sizes_around_a_relabel_tile(la, H, W):
+    """Grids around the 32 x 32 tiles whose relabel passes are skipped when no
+    neighbour changed: the flow and the cut's side equal the oracle's."""
+    rng = np.random.default_rng(100 * H + W)
+    cap = rng.integers(0, 20, (4, H, W)).astype(np.int32)
+    cap[0, :, -1] = 0
+    cap[1, :, 0] = 0
+    cap[2, -1] = 0
+    cap[3, 0] = 0
+    src = (rng.integers(0, 60, (H, W)) * (rng.random((H, W)) < 0.2)).astype(np.int32)
+    snk = (rng.integers(0, 60, (H, W)) * (rng.random((H, W)) < 0.2)).astype(np.int32)
+    expect_same(la, cap, src, snk)

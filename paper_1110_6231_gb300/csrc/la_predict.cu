@@ -681,16 +681,39 @@ __device__ __forceinline__ float2 unpack_bf16(uint32_t u) {
 }
 
 // ctx[i][:] = mean over the rows of segment i of H1 (seg: [I+1] row offsets).
+// ctx is rounded to BF16 next, where another order of the FP32 additions turns
+// a rounding now and then and with it a whole segment's layer 2; so each column
+// is added row by row, by one thread, from 64-row tiles that all 1,024 threads
+// load (the next tile's loads in flight meanwhile).
 __global__ void __launch_bounds__(1024)
 k_segment_mean(const float *__restrict__ Hm, const int *__restrict__ seg, float *__restrict__ ctx) {
-    __shared__ __align__(16) float red[32][H];
-    __shared__ float sums[H];
-    const int i = blockIdx.x;
+    constexpr int kRows = 64;
+    __shared__ __align__(16) float tile[kRows][H];
+    const int i = blockIdx.x, tid = threadIdx.x;
     const int r0 = seg[i], r1 = seg[i + 1];
-    segment_sums(r0, r1, red, sums, [&](int r, int k) {
-        return __ldg(reinterpret_cast<const float4 *>(Hm + (size_t)r * H + k));
-    });
-    if (threadIdx.x < H) ctx[(size_t)i * H + threadIdx.x] = r1 > r0 ? sums[threadIdx.x] / (float)(r1 - r0) : 0.f;
+    const int lr = tid / (H / 4), lk = 4 * (tid % (H / 4));       // rows lr and lr + 32 of a tile
+    float4 next[2];
+    auto load = [&](int r) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            next[h] = r + lr + 32 * h < r1 ? __ldg(reinterpret_cast<const float4 *>(Hm + (size_t)(r + lr + 32 * h) * H + lk))
+                                           : make_float4(0.f, 0.f, 0.f, 0.f);
+    };
+    load(r0);
+    float s = 0.f;
+    for (int r = r0; r < r1; r += kRows) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) *reinterpret_cast<float4 *>(&tile[lr + 32 * h][lk]) = next[h];
+        __syncthreads();
+        load(r + kRows);
+        if (tid < H) {
+            const int rows = min(kRows, r1 - r);
+#pragma unroll 16
+            for (int k = 0; k < rows; ++k) s += tile[k][tid];
+        }
+        __syncthreads();
+    }
+    if (tid < H) ctx[(size_t)i * H + tid] = r1 > r0 ? s / (float)(r1 - r0) : 0.f;
 }
 
 // cseg[i][:] = the pooled path's gradient of segment i: the mean over its

@@ -98,12 +98,15 @@ __global__ void k_mf_init(const int32_t *__restrict__ cap, const int32_t *__rest
 
 // Lock-free push-relabel (Algorithm 4.5 / 4.8), `cycle` passes over the
 // thread's nodes. Loads of state other threads write go to L2 (.cg), so a
-// thread reads some recent value, as the lock-free argument assumes. A pass
-// reads only the excess of an idle node. What a thread pushes into t stays in
-// a register until the end of the launch: every node with a sink arc pushes
-// there, and one atomic each on t's word is a queue of a million at one L2
-// address. With the skipped relabel tiles: 1.31 -> 0.46 ms a 1024 x 1024 cut.
-__global__ void __launch_bounds__(kBlock)
+// thread reads some recent value, as the lock-free argument assumes. What a
+// thread pushes into t stays in a register until the end of the launch: every
+// node with a sink arc pushes there, and one atomic each on t's word is a queue
+// of a million at one L2 address. With the skipped relabel tiles: 1.28 -> 0.42
+// ms a 1024 x 1024 cut. (Excess and height are asked for together: reading the
+// height of active nodes only made a 96 x 101 crossing 5 % slower, one more
+// round trip for each push of its long paths. Eight CTAs an SM, 32 registers:
+// at 40 a 512 x 512 grid no longer has a thread for each node, 6 % slower.)
+__global__ void __launch_bounds__(kBlock, 8)
 k_mf_push(int H, int W, long long *__restrict__ e, int *__restrict__ h, int *__restrict__ cf,
           int *__restrict__ rt, MfCtrl *c, int cycle) {
     const int N = H * W, NV = N + 2;               // |V|: the pixels, s and t
@@ -113,9 +116,8 @@ k_mf_push(int H, int W, long long *__restrict__ e, int *__restrict__ h, int *__r
     for (int it = 0; it < cycle; ++it) {
         for (int u = blockIdx.x * blockDim.x + threadIdx.x; u < N; u += stride) {
             const long long eu = (long long)__ldcg(reinterpret_cast<const unsigned long long *>(e) + u);
-            if (eu <= 0) continue;
             const int hu = h[u];                       // only this thread writes h[u]
-            if (hu >= NV) continue;
+            if (eu <= 0 || hu >= NV) continue;
             // the lowest neighbour over residual arcs (Algorithm 4.5, lines 4-9)
             int hmin = INT_MAX, dmin = -1, cmin = 0;
             const int r = rt[u];                       // only this thread writes rt[u]

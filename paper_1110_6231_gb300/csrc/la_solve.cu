@@ -1041,6 +1041,8 @@ constexpr int kSmallMaxN32 = 224;    // 4 n^2 + 8 n bytes
 // column's cost is kept beside it instead of being read back. Uniform n = 256,
 // costs to 1000: 0.71 -> 0.61 ms a solve; n = 64 unchanged (0.24 ms, more than
 // half of it launches and two host synchronisations).
+// 64-bit values keep one column a lane and read: in fours a scan's 64-bit
+// selects outweigh the reads saved (n = 200: 0.81 -> 1.02 ms).
 struct SmallSched {
     unsigned long long eps[kMaxPhases];    // by value: no copy to wait for
 };
@@ -1142,34 +1144,41 @@ k_small(const int32_t *__restrict__ C, int n, int cmin, uint32_t np1, const __gr
             // best and second best of v(x,y) = (C[x][y] - cmin)(n+1) + q(y) over the row
             const CT *crow = cs + (size_t)row * n;
             ScanResult<V> r{(V)~(V)0, (V)~(V)0, 0, INT_MAX};
-            auto push = [&](int y, uint32_t c, unsigned long long k) {
-                const V cs = (V)c * np1, v = WIDE ? cs + (V)key_q(k) : cs + (V)~(uint32_t)(k >> 32);
-                const bool better = v < r.b1;       // strict: keeps the earliest column
-                const V hi = better ? r.b1 : v;
-                r.b2 = hi < r.b2 ? hi : r.b2;
-                r.c1 = better ? cs : r.c1;
-                r.w = better ? y : r.w;
-                r.b1 = better ? v : r.b1;
-            };
-            if (vec) {
-#pragma unroll 2
-                for (int y = 4 * lane; y < n; y += 128) {
-                    uint32_t c0, c1, c2, c3;
-                    if (C16) {
-                        const ushort4 c = *reinterpret_cast<const ushort4 *>(crow + y);
-                        c0 = c.x, c1 = c.y, c2 = c.z, c3 = c.w;
-                    } else {
-                        const uint4 c = *reinterpret_cast<const uint4 *>(crow + y);
-                        c0 = c.x, c1 = c.y, c2 = c.z, c3 = c.w;
-                    }
-                    const ulonglong2 a = ld_skey2(skey + y), b = ld_skey2(skey + y + 2);
-                    push(y, c0, a.x);
-                    push(y + 1, c1, a.y);
-                    push(y + 2, c2, b.x);
-                    push(y + 3, c3, b.y);
-                }
+            if constexpr (WIDE) {
+                Lane2<V> t;
+                lane2_init(t);
+                for (int y = lane; y < n; y += 32) lane2_push<V>(t, (V)crow[y] * np1 + (V)key_q(vkey[y]), y);
+                r = ScanResult<V>{t.b1, t.b2, t.w1 >= 0 ? (V)crow[t.w1] * np1 : (V)0, t.w1 < 0 ? INT_MAX : t.w1};
             } else {
-                for (int y = lane; y < n; y += 32) push(y, crow[y], vkey[y]);
+                auto push = [&](int y, uint32_t c, unsigned long long k) {
+                    const V cs = (V)c * np1, v = cs + (V)~(uint32_t)(k >> 32);
+                    const bool better = v < r.b1;       // strict: keeps the earliest column
+                    const V hi = better ? r.b1 : v;
+                    r.b2 = hi < r.b2 ? hi : r.b2;
+                    r.c1 = better ? cs : r.c1;
+                    r.w = better ? y : r.w;
+                    r.b1 = better ? v : r.b1;
+                };
+                if (vec) {
+#pragma unroll 2
+                    for (int y = 4 * lane; y < n; y += 128) {
+                        uint32_t c0, c1, c2, c3;
+                        if (C16) {
+                            const ushort4 c = *reinterpret_cast<const ushort4 *>(crow + y);
+                            c0 = c.x, c1 = c.y, c2 = c.z, c3 = c.w;
+                        } else {
+                            const uint4 c = *reinterpret_cast<const uint4 *>(crow + y);
+                            c0 = c.x, c1 = c.y, c2 = c.z, c3 = c.w;
+                        }
+                        const ulonglong2 a = ld_skey2(skey + y), b = ld_skey2(skey + y + 2);
+                        push(y, c0, a.x);
+                        push(y + 1, c1, a.y);
+                        push(y + 2, c2, b.x);
+                        push(y + 3, c3, b.y);
+                    }
+                } else {
+                    for (int y = lane; y < n; y += 32) push(y, crow[y], vkey[y]);
+                }
             }
             warp_merge(r);
             if (r.b2 == (V)~(V)0) r.b2 = r.b1;   // n = 1 cannot reach here; a lone column bids by eps

@@ -1036,7 +1036,7 @@ constexpr int kSmallMaxN32 = 224;    // 4 n^2 + 8 n bytes
 // A bid is a chain of dependent shared-memory reads and instructions of one
 // warp, so both are kept few: with 32-bit values the key is (2^32 - 1 - q) in
 // the high word and the mate in the low one, so that a price is one word and
-// v = c (n+1) + ~hi; where n is a multiple of 4, a lane ranks four columns from
+// v = c (n+1) + ~hi; of 16-bit costs, n a multiple of 4, a lane ranks four columns from
 // one read of their costs and two 16-byte reads of their keys; and the best
 // column's cost is kept beside it instead of being read back. Uniform n = 256,
 // costs to 1000: 0.71 -> 0.61 ms a solve; n = 64 unchanged (0.24 ms, more than
@@ -1091,8 +1091,9 @@ k_small(const int32_t *__restrict__ C, int n, int cmin, uint32_t np1, const __gr
     }
     __syncthreads();
     const volatile unsigned long long *vkey = skey;
-    // four columns a lane: rows of cs then start on 8 (16) bytes; below 128 columns lanes would idle
-    const bool vec = (n & 3) == 0 && n >= 128;
+    // four columns a lane: rows of 16-bit costs then start on 8 bytes; below 128 columns lanes would
+    // idle, and with 32-bit costs the gain is lost (n = 224: 0.65 ms in fours, 0.62 before)
+    const bool vec = C16 && (n & 3) == 0 && n >= 128;
     unsigned long long wins = 0, displaced = 0, chain_max = 0;
     for (int ph = 0; ph < nph; ++ph) {
         const unsigned long long eps = sched.eps[ph];

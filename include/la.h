@@ -511,7 +511,9 @@ la_status la_solve_warm(const int32_t *cost, int32_t n, const void *weights, voi
  * the result is in place. Uses the same la_options / la_stats as
  * la_solve_ex: alpha, eps0, prices_out, scan_budget (0 = 256 n (phases + 1)
  * + 2^22) and profile are honoured; init_prices must be NULL. phase_scans[0]
- * counts the feasibility phase.
+ * counts the feasibility phase. A solve whose price updates would leave the
+ * price field starts again with bids alone; the budget and the counters then
+ * are those of the second attempt (launches counts both).
  */
 la_status la_solve_sparse(const int32_t *row_ptr, const int32_t *cols, const int32_t *costs,
                           int32_t n, int32_t nnz, void *stream, int32_t *match_out,

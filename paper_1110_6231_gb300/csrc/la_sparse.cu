@@ -275,6 +275,22 @@ k_sp_refine(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col
 // no room are read from global memory), eight lanes per column (8..40 arcs a
 // row in the graphs this serves); only the potentials are gathered from L2.
 //
+// The price field. An update lifts every column that lies far from a free
+// column, or reaches none, by K, and K is hops times eps on graphs with long
+// residual paths: prices then climb to many times C~ where bids alone climb to
+// about C~. A lift cut short is no way out: bids alone climb a plateau that
+// updates left in steps of eps. So an update that would lift a price above
+// kFinTop, half of the field, gives the solve up (kGiveUp), and so does a bid
+// that leaves the field; the host then solves again with bids alone, in the
+// refine, as if there were no updates. Emulated bid by bid on the host, largest
+// price / 2^44 with bids alone, with updates without a limit, and as it is
+// now: row x to columns x .. x + 3 at n = 3000, costs to 3.6e8 0.54-0.79,
+// overflow, 0.49; n = 6000, costs to 3e7 0.17-0.20, overflow, 0.18; n = 30000,
+// costs to 2e5 0.02, 0.21, 0.21. What is lost is the first rounds, a few
+// percent of the second attempt. With updates cut short at 2^40 and bids from
+// there on the last graph took 22 million bids, with bids alone 7 million, with
+// updates 0.6. Prices of the graphs timed below stay under 2^32.
+//
 // Measured on GB300, whole solves (mean of 6, ms), from one refine launch per
 // phase: sparse-uniform n = 65536, 33 arcs a row, 193 -> 29; sparse-geometric
 // n = 16384, 36 arcs a row, 242 -> 94. There the 50 updates take 58 ms (150
@@ -295,6 +311,8 @@ constexpr int kFinMetaCap = 4096;                           // columns per CTA w
 constexpr int kFinSmem = 200 * 1024;
 constexpr unsigned long long kFar = 1ull << 62;             // no path found yet
 constexpr int kFinBids = 256;                               // bids of a warp's chain in one round
+constexpr unsigned long long kFinTop = kQMax / 2;           // no update lifts a price above it
+constexpr int kGiveUp = -1;                                 // status: solve again with bids alone
 
 __device__ __forceinline__ unsigned long long min_u64_group(unsigned long long v) {
 #pragma unroll
@@ -551,16 +569,19 @@ k_sp_finish(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col
             if (!grid_barrier(&fin->bar, &ctrl->status, &s_ok)) return;
             if (it == 0) continue;
             lim = *reinterpret_cast<volatile unsigned long long *>(&fin->need[slot]);
-            if ( *reinterpret_cast<volatile int *>(&fin->changed[slot]) == 0) break;
+            if (*reinterpret_cast<volatile int *>(&fin->changed[slot]) == 0) break;
         }
         ++updates;
         // lim is now the largest distance of a free row: the level K
-        if (lim >= kFar && gtid == 0) sp_set_status(ctrl, LA_ERR_INFEASIBLE);
+        if (gtid == 0) {
+            const unsigned long long qmax = *reinterpret_cast<volatile unsigned long long *>(&fin->qmax[par]);
+            if (lim >= kFar) sp_set_status(ctrl, LA_ERR_INFEASIBLE);
+            else if (qmax + lim > kFinTop) sp_set_status(ctrl, kGiveUp);
+        }
         const int count = *reinterpret_cast<volatile int *>(&fin->count[par]);
         if (!grid_barrier(&fin->bar, &ctrl->status, &s_ok)) return;
         if (*reinterpret_cast<volatile int *>(&ctrl->status) != 0) break;
-        const unsigned long long qmax = *reinterpret_cast<volatile unsigned long long *>(&fin->qmax[par]);
-        const unsigned long long K = min(lim, qlim > qmax ? qlim - qmax : 0ull);
+        const unsigned long long K = lim;
         for (int y = gtid; y < n && K > 0; y += gthreads) {
             const unsigned long long k = __ldcg(key + y);
             const unsigned long long q = key_q(k), s = __ldcg(pot + y), nq = s < q + K ? max(s, q) : q + K;
@@ -806,50 +827,70 @@ static la_status sparse_locked(const int32_t *row_ptr, const int32_t *cols, cons
                                                               : 256ull * n * (sched.size() + 1) + (1ull << 22);
     const int grid = std::max(1, std::min(w.num_sms * w.occ, (n + kBlock / 32 - 1) / (kBlock / 32)));
     if (profile) LA_SCK(cudaEventRecord(w.ev[0], s));
-    const int hand_free = sp_hand_free(n);
     const unsigned long long qinf = 4ull * (unsigned long long)n + 4;
-    // feasibility phase: zero costs, eps = 1, prices from 0
-    k_sp_reset<<<sg, kBlock, 0, s>>>(w.key, w.qm, n, qlim, w.ctrl, w.fin, 0, 0, 1);
-    k_sp_refine<true><<<grid, kBlock, 0, s>>>(row_ptr, cols, costs, n, c0.cmin, (uint32_t)np1, 1ull, qlim,
-                                              qinf, w.key, w.qm, w.ctrl, budget, w.fin, hand_free);
-    LA_SCK(launch_finish<true>(s, w, row_ptr, cols, costs, n, c0.cmin, (uint32_t)np1, 1ull, qlim, qinf, budget));
-    launches += 3;
-    // cost phases (Algorithm 5.0), from zero prices again
+    // with end-of-phase updates; if those leave the price field, again with bids alone
+    Ctrl c1;
     int ph = 0;
-    for (; ph < (int)sched.size(); ++ph) {
-        const int slot = ph & 1;
-        if (ph > 0) {
-            k_sp_qmin<<<sg, kBlock, 0, s>>>(w.key, n, w.ctrl, slot);
+    bool alone = false;
+    for (;; alone = true) {
+        const int hand_free = alone ? -1 : sp_hand_free(n);
+        if (alone) {
+            init.cmin = c0.cmin;
+            init.cmax = c0.cmax;
+            *w.h_ctrl = init;
+            LA_SCK(cudaMemcpyAsync(w.ctrl, w.h_ctrl, sizeof(Ctrl), cudaMemcpyHostToDevice, s));
+            LA_SCK(cudaMemsetAsync(w.fin, 0, sizeof(FinCtrl), s));
+        }
+        // feasibility phase: zero costs, eps = 1, prices from 0
+        k_sp_reset<<<sg, kBlock, 0, s>>>(w.key, w.qm, n, qlim, w.ctrl, w.fin, 0, 0, 1);
+        k_sp_refine<true><<<grid, kBlock, 0, s>>>(row_ptr, cols, costs, n, c0.cmin, (uint32_t)np1, 1ull, qlim,
+                                                  qinf, w.key, w.qm, w.ctrl, budget, w.fin, hand_free);
+        launches += 2;
+        if (!alone) {
+            LA_SCK(launch_finish<true>(s, w, row_ptr, cols, costs, n, c0.cmin, (uint32_t)np1, 1ull, qlim, qinf,
+                                       budget));
             ++launches;
         }
-        k_sp_reset<<<sg, kBlock, 0, s>>>(w.key, w.qm, n, qlim, w.ctrl, w.fin, slot, ph + 1, ph == 0);
-        k_sp_refine<false><<<grid, kBlock, 0, s>>>(row_ptr, cols, costs, n, c0.cmin, (uint32_t)np1, sched[ph],
-                                                   qlim, ~0ull, w.key, w.qm, w.ctrl, budget, w.fin, hand_free);
-        LA_SCK(launch_finish<false>(s, w, row_ptr, cols, costs, n, c0.cmin, (uint32_t)np1, sched[ph], qlim, ~0ull,
-                                    budget));
-        launches += 3;
-    }
-    if (profile) LA_SCK(cudaEventRecord(w.ev[1], s));
-    const int fslot = ph & 1;
-    if (prices_out) {
-        k_sp_qmin<<<sg, kBlock, 0, s>>>(w.key, n, w.ctrl, fslot);
+        // cost phases (Algorithm 5.0), from zero prices again
+        for (ph = 0; ph < (int)sched.size(); ++ph) {
+            const int slot = ph & 1;
+            if (ph > 0) {
+                k_sp_qmin<<<sg, kBlock, 0, s>>>(w.key, n, w.ctrl, slot);
+                ++launches;
+            }
+            k_sp_reset<<<sg, kBlock, 0, s>>>(w.key, w.qm, n, qlim, w.ctrl, w.fin, slot, ph + 1, ph == 0);
+            k_sp_refine<false><<<grid, kBlock, 0, s>>>(row_ptr, cols, costs, n, c0.cmin, (uint32_t)np1, sched[ph],
+                                                       qlim, ~0ull, w.key, w.qm, w.ctrl, budget, w.fin, hand_free);
+            launches += 2;
+            if (!alone) {
+                LA_SCK(launch_finish<false>(s, w, row_ptr, cols, costs, n, c0.cmin, (uint32_t)np1, sched[ph], qlim,
+                                            ~0ull, budget));
+                ++launches;
+            }
+        }
+        if (profile) LA_SCK(cudaEventRecord(w.ev[1], s));
+        const int fslot = ph & 1;
+        if (prices_out) {
+            k_sp_qmin<<<sg, kBlock, 0, s>>>(w.key, n, w.ctrl, fslot);
+            ++launches;
+        }
+        LA_SCK(cudaMemsetAsync(cost_out, 0, sizeof(int64_t), s));
+        k_sp_finalize<<<sg, kBlock, 0, s>>>(row_ptr, cols, costs, n, w.key, match_out,
+                                            reinterpret_cast<long long *>(cost_out),
+                                            reinterpret_cast<long long *>(prices_out), w.ctrl, fslot);
         ++launches;
+        LA_SCK(cudaGetLastError());
+        LA_SCK(cudaMemcpyAsync(w.h_ctrl, w.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s));
+        LA_SCK(cudaStreamSynchronize(s));
+        c1 = *w.h_ctrl;
+        if (alone || (c1.status != kGiveUp && c1.status != LA_ERR_OVERFLOW)) break;
     }
-    LA_SCK(cudaMemsetAsync(cost_out, 0, sizeof(int64_t), s));
-    k_sp_finalize<<<sg, kBlock, 0, s>>>(row_ptr, cols, costs, n, w.key, match_out,
-                                        reinterpret_cast<long long *>(cost_out),
-                                        reinterpret_cast<long long *>(prices_out), w.ctrl, fslot);
-    ++launches;
-    LA_SCK(cudaGetLastError());
-    LA_SCK(cudaMemcpyAsync(w.h_ctrl, w.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s));
-    LA_SCK(cudaStreamSynchronize(s));
-    const Ctrl c1 = *w.h_ctrl;
     stats.phases = (int64_t)sched.size();
     stats.scans = (int64_t)c1.scans;
     stats.wins = (int64_t)c1.wins;
     stats.displaced = (int64_t)c1.displaced;
     stats.launches = launches;
-    stats.refine_launches = 2 * ((int64_t)sched.size() + 1);
+    stats.refine_launches = (alone ? 1 : 2) * ((int64_t)sched.size() + 1);
     stats.price_updates = (int64_t)c1.pu_updates;
     stats.price_update_sweeps = (int64_t)c1.pu_iters;
     stats.max_chain = (int64_t)c1.max_chain;

@@ -1,0 +1,39 @@
+"""Sparse graphs whose scaled costs come near the top of the price field.
+
+la_solve_sparse accepts every graph with (n + 1)(max C - min C) < 2^40. On
+graphs whose residual paths are long, a price update's distances are many
+times that range: it must not use up the 2^44 price field, so that such a
+graph ends in its optimum, as with bids alone, and not in LA_ERR_OVERFLOW. Whole numbers: every comparison is exact."""
+
+import numpy as np
+import pytest
+
+from test_gpu_sparse import expect_same, gpu_solve, la  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+def band(n, hi, seed, width=4):
+    """Row x has arcs to columns x .. x + width - 1 (mod n), costs uniform on [0, hi]."""
+    rng = np.random.default_rng(seed)
+    cols = (np.arange(n)[:, None] + np.arange(width)) % n
+    return np.arange(n + 1) * width, cols.ravel(), rng.integers(0, hi + 1, n * width)
+
+
+@pytest.mark.parametrize("seed", [1, 2, 3])
+@pytest.mark.parametrize("n,hi", [(3000, 10**8), (3000, 360_000_000), (6000, 3 * 10**7)])
+def test_long_paths_near_the_top_of_the_range(la, n, hi, seed):  # noqa: F811
+    rp, cols, costs = band(n, hi, seed)
+    assert (n + 1) * int(costs.max() - costs.min()) < 1 << 40
+    assert expect_same(la, rp, cols, costs) is not None
+
+
+def test_the_scan_budget_holds_when_a_solve_starts_again(la):  # noqa: F811
+    """At this range the updates are given up and the solve starts again with
+    bids alone; it still stops at the budget, and the next call is clean."""
+    g = band(3000, 360_000_000, 4)
+    need = gpu_solve(la, *g).stats["scans"]
+    got = gpu_solve(la, *g, scan_budget=need // 8)
+    assert got.stats["status"] == la.LA_ERR_ITER_LIMIT
+    assert got.stats["scans"] < need
+    assert expect_same(la, *g) is not None

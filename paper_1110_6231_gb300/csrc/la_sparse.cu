@@ -300,6 +300,19 @@ k_sp_refine(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col
 // 256 and 1024 bids a round: 107, 88 and 95 ms (and 36, 29, 31 on the uniform
 // graph): short chains do not reach the end of their path, long ones are rows
 // whose path was taken, in a price war that the next update ends sooner.
+//
+// Paths longer than 256 need longer chains, or each round moves every row 256
+// columns on and pays a whole update for it: a chain may take as many bids as
+// the update took sweeps (about the columns of its longest path, and a third
+// of its time). And where paths lead through most of the graph bids alone are
+// faster: kGiveUp if a phase's first update leaves a free row that has reached
+// no free column after kFinReach sweeps (cycles of rows of two arcs: 150 to
+// 2,000; random and search-window graphs of three arcs a row and more, n = 600
+// to 65536: at most 28; row x to columns x .. x + 3: 76), or is not done after
+// n / 2 (1,024 to 16,384; there at most n / 5). n = 30000, row x to columns x
+// .. x + d - 1, ms, with bids alone, with 256 bids a chain (emulated), now:
+// d = 2 230-960, 63,000, 310-440; d = 4 1,700-6,000, 3,000, 190-290; d = 8
+// 2,300-5,300, 450 (n = 20000), 170-200.
 constexpr int kFinBlock = 1024;
 constexpr int kFinLanes = 8;                                // lanes per column in a sweep
 constexpr int kFinPerWarp = 32 / kFinLanes;
@@ -310,7 +323,8 @@ constexpr int kFinMinCols = 16;                             // columns per CTA a
 constexpr int kFinMetaCap = 4096;                           // columns per CTA with cached arcs
 constexpr int kFinSmem = 200 * 1024;
 constexpr unsigned long long kFar = 1ull << 62;             // no path found yet
-constexpr int kFinBids = 256;                               // bids of a warp's chain in one round
+constexpr int kFinBids = 256;                               // bids of a warp's chain in one round, at least
+constexpr unsigned kFinReach = 128;                         // sweeps until every free row has reached a free column
 constexpr unsigned long long kFinTop = kQMax / 2;           // no update lifts a price above it
 constexpr int kGiveUp = -1;                                 // status: solve again with bids alone
 
@@ -359,6 +373,7 @@ k_sp_finish(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col
     int2 *s_at = reinterpret_cast<int2 *>(s_q + meta_cap);                         // [meta_cap] first arc, padded count
     unsigned *s_cy = reinterpret_cast<unsigned *>(s_at + meta_cap);                // [meta_cap] cost of the matched arc
     int2 *s_arc = reinterpret_cast<int2 *>(s_cy + ((meta_cap + 1) & ~1));          // [arc_cap] column, cost - cmin
+    const unsigned max_first = min(16384u, max(1024u, (unsigned)n / 2));
     unsigned long long sweeps = 0;
     unsigned long long wins = 0, displaced = 0, total = 0, longest = 0, updates = 0;
     for (int round = 0;; ++round) {
@@ -436,6 +451,8 @@ k_sp_finish(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col
         // changed nothing here; an epoch in which no CTA changed anything
         // proves the fixed point.
         unsigned long long lim = kFar;     // no column farther than this matters
+        unsigned used = 0;                 // sweeps of this update, at most (the same for every CTA)
+        bool settled = false;
         for (int it = 0; it <= n + 1; ++it) {
             const int slot = it % 3;
             bool any = false;
@@ -473,6 +490,7 @@ k_sp_finish(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col
                 __syncthreads();
             }
             const int most = it < 2 ? kFinFirst : kFinSweeps;
+            used += most;
             for (int sw = 0, quiet = 0; sw < most && quiet < kFinQuiet; ++sw) {
                 bool fell = false;
                 for (int j0 = warp * kFinPerWarp; j0 < mine; j0 += (kFinBlock / 32) * kFinPerWarp) {
@@ -569,13 +587,18 @@ k_sp_finish(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col
             if (!grid_barrier(&fin->bar, &ctrl->status, &s_ok)) return;
             if (it == 0) continue;
             lim = *reinterpret_cast<volatile unsigned long long *>(&fin->need[slot]);
-            if (*reinterpret_cast<volatile int *>(&fin->changed[slot]) == 0) break;
+            if (*reinterpret_cast<volatile int *>(&fin->changed[slot]) == 0) {
+                settled = true;
+                break;
+            }
+            if (updates == 0 && used > (lim >= kFar ? kFinReach : max_first)) break;   // paths too long for updates
         }
         ++updates;
         // lim is now the largest distance of a free row: the level K
         if (gtid == 0) {
             const unsigned long long qmax = *reinterpret_cast<volatile unsigned long long *>(&fin->qmax[par]);
-            if (lim >= kFar) sp_set_status(ctrl, LA_ERR_INFEASIBLE);
+            if (!settled) sp_set_status(ctrl, kGiveUp);
+            else if (lim >= kFar) sp_set_status(ctrl, LA_ERR_INFEASIBLE);
             else if (qmax + lim > kFinTop) sp_set_status(ctrl, kGiveUp);
         }
         const int count = *reinterpret_cast<volatile int *>(&fin->count[par]);
@@ -598,23 +621,25 @@ k_sp_finish(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col
             }
         }
         if (!grid_barrier(&fin->bar, &ctrl->status, &s_ok)) return;
-        // the free rows bid, one warp per row, spread over the SMs first
+        // the free rows bid, one warp per row, spread over the SMs first; a chain may be as long as the paths
+        const unsigned most_bids = max((unsigned)kFinBids, used);
         for (int i = warp * gridDim.x + blockIdx.x; i < count; i += gridDim.x * (blockDim.x >> 5)) {
             int row = __ldcg(rows + i);
             unsigned steps = 0;
-            while (row >= 0 && steps < (unsigned)kFinBids) {
-                ++steps;
-                row = sp_bid<ZERO>(row_ptr, cols, costs, n, cmin, np1, eps, qlim, qinf, key, qm, ctrl, row, lane, wins,
-                                   displaced);
+            while (row >= 0 && steps < most_bids) {
+                unsigned now = 0;      // the scans are counted every kFinBids bids
+                while (row >= 0 && now < (unsigned)kFinBids) {
+                    ++now;
+                    row = sp_bid<ZERO>(row_ptr, cols, costs, n, cmin, np1, eps, qlim, qinf, key, qm, ctrl, row, lane,
+                                       wins, displaced);
+                }
+                steps += now;
+                if (lane == 0 && atomicAdd(&ctrl->scans, (unsigned long long)now) + now > budget)
+                    sp_set_status(ctrl, LA_ERR_ITER_LIMIT);
             }
             if (row == kMatched && lane == 0) atomicSub(&fin->free_rows, 1);
             total += steps;
             longest = max(longest, (unsigned long long)steps);
-            unsigned long long sc = 0;
-            if (lane == 0) {
-                sc = atomicAdd(&ctrl->scans, (unsigned long long)steps) + steps;
-                if (sc > budget) sp_set_status(ctrl, LA_ERR_ITER_LIMIT);
-            }
             if (row == kFailed) break;
         }
         if (!grid_barrier(&fin->bar, &ctrl->status, &s_ok)) return;

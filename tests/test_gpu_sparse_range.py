@@ -8,6 +8,8 @@ graph ends in its optimum, as with bids alone, and not in LA_ERR_OVERFLOW. Whole
 import numpy as np
 import pytest
 
+import oracle
+
 from test_gpu_sparse import expect_same, gpu_solve, la  # noqa: F401
 
 pytestmark = pytest.mark.gpu
@@ -37,3 +39,18 @@ def test_the_scan_budget_holds_when_a_solve_starts_again(la):  # noqa: F811
     assert got.stats["status"] == la.LA_ERR_ITER_LIMIT
     assert got.stats["scans"] < need
     assert expect_same(la, *g) is not None
+
+
+@pytest.mark.parametrize("width,hi", [(2, 1000), (4, 10_000), (8, 1000)])
+def test_long_paths_take_few_rounds(la, width, hi):  # noqa: F811
+    """Residual paths of thousands of columns: a round's chains must follow
+    them to their end, not a fixed number of columns a round (then one update
+    for every 256 columns of path, hundreds in all). The prices certify the
+    matching."""
+    rp, cols, costs = band(30_000, hi, 5, width)
+    sol = gpu_solve(la, rp, cols, costs, want_prices=True)
+    assert sol.stats["status"] == la.LA_OK
+    match = sol.match.cpu().numpy()
+    assert oracle.sparse_check_matching(rp, cols, costs, match, sol.cost) == 0
+    assert oracle.sparse_check_eps_cs(rp, cols, costs, match, sol.prices.cpu().numpy(), 1) == 0
+    assert sol.stats["price_updates"] <= 5 * (sol.stats["phases"] + 1)

@@ -756,6 +756,18 @@ int sp_hand_free(int n) {
     return std::max(8, n / 64);
 }
 
+// Cost phases without the end-of-phase kernel: where a phase is shorter than
+// its launch and a few grid barriers, and where rows have two arcs on average,
+// so that residual paths are long and hardly branch. ms with the kernel in
+// every phase, without: 9 arcs a row, n = 50 0.58, 0.37; n = 200 0.79, 0.54;
+// n = 500 1.2, 1.2 (n = 1000: 2.0, 3.3 without); search windows, n = 256 0.63,
+// 0.46. Two arcs a row, n = 600 1.4, 0.87; n = 65536 20-41, 14-22; cycles of
+// two arcs a row, n = 2500 83, 18 (three arcs a row: 3.6, 6.4).
+// The feasibility phase keeps the kernel, which finds in one update what takes
+// bids alone a price war of 4n steps (12 rows on 11 columns among n = 600:
+// 0.3 and 21.6 ms).
+bool sp_bids_alone(int n, int nnz) { return n <= 512 || (int64_t)nnz * 2 <= (int64_t)n * 5; }
+
 // The end-of-phase kernel on a co-resident grid: one CTA per SM, fewer when
 // the graph has fewer columns than the grid has lane groups.
 template <bool ZERO>
@@ -857,8 +869,10 @@ static la_status sparse_locked(const int32_t *row_ptr, const int32_t *cols, cons
     Ctrl c1;
     int ph = 0;
     bool alone = false;
+    const bool short_solve = sp_bids_alone(n, nnz);
     for (;; alone = true) {
-        const int hand_free = alone ? -1 : sp_hand_free(n);
+        const int hand_free = alone ? -1 : sp_hand_free(n);          // of the feasibility phase
+        const bool updates = !alone && !short_solve;                 // of the cost phases
         if (alone) {
             init.cmin = c0.cmin;
             init.cmax = c0.cmax;
@@ -885,9 +899,10 @@ static la_status sparse_locked(const int32_t *row_ptr, const int32_t *cols, cons
             }
             k_sp_reset<<<sg, kBlock, 0, s>>>(w.key, w.qm, n, qlim, w.ctrl, w.fin, slot, ph + 1, ph == 0);
             k_sp_refine<false><<<grid, kBlock, 0, s>>>(row_ptr, cols, costs, n, c0.cmin, (uint32_t)np1, sched[ph],
-                                                       qlim, ~0ull, w.key, w.qm, w.ctrl, budget, w.fin, hand_free);
+                                                       qlim, ~0ull, w.key, w.qm, w.ctrl, budget, w.fin,
+                                                       updates ? hand_free : -1);
             launches += 2;
-            if (!alone) {
+            if (updates) {
                 LA_SCK(launch_finish<false>(s, w, row_ptr, cols, costs, n, c0.cmin, (uint32_t)np1, sched[ph], qlim,
                                             ~0ull, budget));
                 ++launches;
@@ -915,7 +930,7 @@ static la_status sparse_locked(const int32_t *row_ptr, const int32_t *cols, cons
     stats.wins = (int64_t)c1.wins;
     stats.displaced = (int64_t)c1.displaced;
     stats.launches = launches;
-    stats.refine_launches = (alone ? 1 : 2) * ((int64_t)sched.size() + 1);
+    stats.refine_launches = (alone || short_solve ? 1 : 2) * ((int64_t)sched.size() + 1) + (short_solve && !alone);
     stats.price_updates = (int64_t)c1.pu_updates;
     stats.price_update_sweeps = (int64_t)c1.pu_iters;
     stats.max_chain = (int64_t)c1.max_chain;

@@ -9,6 +9,7 @@ import numpy as np
 import pytest
 
 import oracle
+from paper_1110_6231_gb300 import synth
 
 from test_gpu_sparse import expect_same, gpu_solve, la  # noqa: F401
 
@@ -54,3 +55,14 @@ def test_long_paths_take_few_rounds(la, width, hi):  # noqa: F811
     assert oracle.sparse_check_matching(rp, cols, costs, match, sol.cost) == 0
     assert oracle.sparse_check_eps_cs(rp, cols, costs, match, sol.prices.cpu().numpy(), 1) == 0
     assert sol.stats["price_updates"] <= 5 * (sol.stats["phases"] + 1)
+
+
+@pytest.mark.parametrize("n", [511, 512, 513])
+@pytest.mark.parametrize("degree", [1, 2, 8])
+def test_both_sides_of_the_line_for_bids_alone(la, n, degree):  # noqa: F811
+    """Up to 512 rows, and up to five arcs for two rows, the cost phases run
+    without updates; one row or one arc more and they have them."""
+    rp, cols, costs = synth.sparse_uniform(n, degree, n)
+    sol = expect_same(la, rp, cols, costs)
+    updates = n > 512 and 2 * cols.size > 5 * n
+    assert sol.stats["refine_launches"] == (2 if updates else 1) * (sol.stats["phases"] + 1) + (not updates)

@@ -505,9 +505,10 @@ la_status la_solve_warm(const int32_t *cost, int32_t n, const void *weights, voi
  *   cost_out  device int64[1]: the optimal total cost.
  * Returns LA_OK; LA_ERR_INVALID for malformed CSR arrays (checked on the
  * device before any solving); LA_ERR_INFEASIBLE when no perfect matching
- * exists (a row or column without arcs, or a price drop in a first refine
- * phase on zero costs beyond what a feasible graph allows: 4n + 4, against
- * the bound (2n - 1) eps of cost scaling); else as la_solve. Blocks until
+ * exists (a row or column without arcs; or, in a first phase on zero costs, a
+ * price drop by bids alone beyond what a feasible graph allows: 4n + 4,
+ * against the bound (2n - 1) eps of cost scaling; or a free row that reaches
+ * no free column in the residual graph); else as la_solve. Blocks until
  * the result is in place. Uses the same la_options / la_stats as
  * la_solve_ex: alpha, eps0, prices_out, scan_budget (0 = 256 n (phases + 1)
  * + 2^22) and profile are honoured; init_prices must be NULL. phase_scans[0]

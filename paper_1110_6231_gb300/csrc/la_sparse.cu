@@ -22,10 +22,16 @@
 //    price-drop bound of cost scaling (the path argument behind Lemma 5.6's
 //    use of eps-optimality: a column relabelled while it holds excess lies on
 //    an alternating path to a free column, of at most 2n - 1 arcs) keeps every
-//    price within (eps + 0)(2n - 1) of its start. A drop beyond 4n + 4 in that
-//    phase therefore proves that no perfect matching exists
-//    (LA_ERR_INFEASIBLE); otherwise prices are reset and the cost phases run
-//    on a graph known to be feasible.
+//    price within (eps + 0)(2n - 1) of its start while bids alone move the
+//    prices. A bid beyond 4n + 4 in the refine, which runs from zero prices,
+//    therefore proves that no perfect matching exists (LA_ERR_INFEASIBLE).
+//    The updates that end the phase (k_sp_finish) also lift columns that reach
+//    no free column, which that argument says nothing about, so there no price
+//    decides: a free row that reaches no free column in the residual graph has
+//    no augmenting path, and the matching cannot become perfect
+//    (LA_ERR_INFEASIBLE too); while every free row reaches one the rounds go
+//    on. Then prices are reset and the cost phases run on a graph known to be
+//    feasible.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -264,7 +270,7 @@ k_sp_refine(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col
 // starts a shortest path, and its bids walk along it (l = 0 up to ties)
 // unless the paths of two rows cross; such rows go into the next round. A
 // free row that reaches no free column has no augmenting path: no perfect
-// matching exists.
+// matching exists (the only test for that here; no price bound).
 //
 // Two bounds keep the sweeps short. The free rows' distances at the
 // potentials so far bound K from above: a column farther than that is not
@@ -352,7 +358,7 @@ template <bool ZERO>
 __global__ void __launch_bounds__(kFinBlock)
 k_sp_finish(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ cols,
             const int32_t *__restrict__ costs, int n, int cmin, uint32_t np1, unsigned long long eps,
-            unsigned long long qlim, unsigned long long qinf, unsigned long long *__restrict__ key,
+            unsigned long long qlim, unsigned long long *__restrict__ key,
             unsigned long long *__restrict__ qm, unsigned long long *__restrict__ pot, int *__restrict__ rowcol,
             int *__restrict__ rows, Ctrl *__restrict__ ctrl, unsigned long long budget, FinCtrl *__restrict__ fin,
             int meta_cap, int arc_cap) {
@@ -630,7 +636,7 @@ k_sp_finish(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col
                 unsigned now = 0;      // the scans are counted every kFinBids bids
                 while (row >= 0 && now < (unsigned)kFinBids) {
                     ++now;
-                    row = sp_bid<ZERO>(row_ptr, cols, costs, n, cmin, np1, eps, qlim, qinf, key, qm, ctrl, row, lane,
+                    row = sp_bid<ZERO>(row_ptr, cols, costs, n, cmin, np1, eps, qlim, ~0ull, key, qm, ctrl, row, lane,
                                        wins, displaced);
                 }
                 steps += now;
@@ -773,7 +779,7 @@ bool sp_bids_alone(int n, int nnz) { return n <= 512 || (int64_t)nnz * 2 <= (int
 template <bool ZERO>
 cudaError_t launch_finish(cudaStream_t s, SparseWorkspace &w, const int32_t *row_ptr, const int32_t *cols,
                           const int32_t *costs, int n, int cmin, uint32_t np1, unsigned long long eps,
-                          unsigned long long qlim, unsigned long long qinf, unsigned long long budget) {
+                          unsigned long long qlim, unsigned long long budget) {
     const int grid = std::max(1, std::min(w.num_sms, (n + kFinMinCols - 1) / kFinMinCols));
     // shared memory: what this graph needs, up to kFinSmem
     const int chunks = (n + kFinMinCols - 1) / kFinMinCols;
@@ -784,7 +790,7 @@ cudaError_t launch_finish(cudaStream_t s, SparseWorkspace &w, const int32_t *row
         cudaFuncSetAttribute(k_sp_finish<ZERO>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFinSmem);
     if (e != cudaSuccess) return e;
     void *args[] = {(void *)&row_ptr, (void *)&cols, (void *)&costs, (void *)&n, (void *)&cmin, (void *)&np1,
-                    (void *)&eps, (void *)&qlim, (void *)&qinf, (void *)&w.key, (void *)&w.qm, (void *)&w.pot,
+                    (void *)&eps, (void *)&qlim, (void *)&w.key, (void *)&w.qm, (void *)&w.pot,
                     (void *)&w.rowcol, (void *)&w.rows, (void *)&w.ctrl, (void *)&budget, (void *)&w.fin,
                     (void *)&meta_cap, (void *)&arc_cap};
     return cudaLaunchCooperativeKernel((const void *)k_sp_finish<ZERO>, dim3(grid), dim3(kFinBlock), args, kFinSmem, s);
@@ -886,8 +892,7 @@ static la_status sparse_locked(const int32_t *row_ptr, const int32_t *cols, cons
                                                   qinf, w.key, w.qm, w.ctrl, budget, w.fin, hand_free);
         launches += 2;
         if (!alone) {
-            LA_SCK(launch_finish<true>(s, w, row_ptr, cols, costs, n, c0.cmin, (uint32_t)np1, 1ull, qlim, qinf,
-                                       budget));
+            LA_SCK(launch_finish<true>(s, w, row_ptr, cols, costs, n, c0.cmin, (uint32_t)np1, 1ull, qlim, budget));
             ++launches;
         }
         // cost phases (Algorithm 5.0), from zero prices again
@@ -904,7 +909,7 @@ static la_status sparse_locked(const int32_t *row_ptr, const int32_t *cols, cons
             launches += 2;
             if (updates) {
                 LA_SCK(launch_finish<false>(s, w, row_ptr, cols, costs, n, c0.cmin, (uint32_t)np1, sched[ph], qlim,
-                                            ~0ull, budget));
+                                            budget));
                 ++launches;
             }
         }

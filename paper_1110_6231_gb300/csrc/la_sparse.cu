@@ -278,8 +278,19 @@ k_sp_refine(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col
 // (min(D, K) is the same). And the CTAs sweep on without waiting for each
 // other; grid barriers come once an epoch. A CTA keeps the arcs of its
 // columns' rows in shared memory for a round (8 bytes an arc, rows that find
-// no room are read from global memory), eight lanes per column (8..40 arcs a
-// row in the graphs this serves); only the potentials are gathered from L2.
+// no room are read from global memory and leave the room to shorter ones),
+// eight lanes per column (8..40 arcs a row in the graphs this serves); only
+// the potentials are gathered from L2.
+//
+// A row of more than kFinLongRow arcs would keep its eight lanes through 16
+// and more rounds of gathers while every other CTA waits at the barrier, and
+// would fill the shared memory. Such rows are listed instead, and the CTA's 32
+// warps read them in segments of kFinSeg arcs. Whole solves, ms, with bids
+// alone, with eight lanes for every row, now: 9 arcs a row and 20 rows of 8,192
+// at n = 8192 28, 39, 23; 16 rows of 2,048 at n = 2048 5.3-7.1, 9.9, 5.8-8.2; one
+// of 16,384 at n = 16384 -, 64, 35; 4 rows of 20,000 at n = 65536 150-195
+// and 49-58, 65 arcs a row there 223-263 and 60-66, 9 arcs a row at n = 10^6
+// 2,560 and 1,610 (bids alone and now).
 //
 // The price field. An update lifts every column that lies far from a free
 // column, or reaches none, by K, and K is hops times eps on graphs with long
@@ -327,6 +338,9 @@ constexpr int kFinSweeps = 16;                              // sweeps of an epoc
 constexpr int kFinQuiet = 3;                                // ... and sweeps without a change that end it
 constexpr int kFinMinCols = 16;                             // columns per CTA at least
 constexpr int kFinMetaCap = 4096;                           // columns per CTA with cached arcs
+constexpr int kFinLongRow = 512;                            // rows of more arcs are read by whole warps
+constexpr int kFinLongRows = 256;                           // ... so many of them per CTA
+constexpr int kFinSeg = 512;                                // ... in segments of so many arcs
 constexpr int kFinSmem = 200 * 1024;
 constexpr unsigned long long kFar = 1ull << 62;             // no path found yet
 constexpr int kFinBids = 256;                               // bids of a warp's chain in one round, at least
@@ -363,7 +377,12 @@ k_sp_finish(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col
             int *__restrict__ rows, Ctrl *__restrict__ ctrl, unsigned long long budget, FinCtrl *__restrict__ fin,
             int meta_cap, int arc_cap) {
     extern __shared__ unsigned long long fin_smem[];
-    __shared__ int s_ok, s_used;
+    __shared__ int s_ok, s_used, s_nlong;
+    // long rows of this CTA's columns: column, first arc, arcs, segments up to and with this row, cost of the
+    // matched arc, price, S, and the best arc's value in a sweep
+    __shared__ int l_y[kFinLongRows], l_b[kFinLongRows], l_deg[kFinLongRows], l_end[kFinLongRows];
+    __shared__ unsigned l_cy[kFinLongRows];
+    __shared__ unsigned long long l_q[kFinLongRows], l_cur[kFinLongRows], l_best[kFinLongRows];
     if (threadIdx.x == 0) s_ok = 1;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int gtid = blockIdx.x * blockDim.x + tid, gthreads = gridDim.x * blockDim.x;
@@ -409,8 +428,8 @@ k_sp_finish(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col
         if (!grid_barrier(&fin->bar, &ctrl->status, &s_ok)) return;
         for (int x = gtid; x < n; x += gthreads)
             if (__ldcg(rowcol + x) < 0) rows[atomicAdd(&fin->count[par], 1)] = x;
-        // the arcs of this CTA's columns' rows into shared memory
-        if (tid == 0) s_used = 0;
+        // the arcs of this CTA's columns' rows into shared memory, long rows into their list
+        if (tid == 0) s_used = s_nlong = 0;
         __syncthreads();
         for (int j0 = warp * kFinPerWarp; j0 < mine; j0 += (kFinBlock / 32) * kFinPerWarp) {
             const int j = j0 + lane / kFinLanes;
@@ -423,11 +442,30 @@ k_sp_finish(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col
                     deg = __ldg(row_ptr + x + 1) - b;
                 }
             }
-            const int pad = (deg + kFinLanes - 1) / kFinLanes * kFinLanes;
-            int at = 0;
-            if (sub == 0 && pad) at = atomicAdd(&s_used, pad);
+            int at = -1;                           // place of the arcs; -2: in the list
+            if (sub == 0 && deg > kFinLongRow) {
+                const int k = atomicAdd(&s_nlong, 1);
+                if (k < kFinLongRows) {
+                    at = -2;
+                    l_y[k] = y;
+                    l_b[k] = b;
+                    l_deg[k] = deg;
+                    l_cy[k] = 0xffffffffu;
+                    l_q[k] = key_q(__ldcg(key + y));
+                    l_cur[k] = l_best[k] = kFar;
+                }
+            } else if (sub == 0 && deg && j < meta_cap) {
+                const int pad = (deg + kFinLanes - 1) / kFinLanes * kFinLanes;
+                if (*(volatile int *)&s_used + pad <= arc_cap) {
+                    at = atomicAdd(&s_used, pad);
+                    if (at + pad > arc_cap) {      // others took the room: leave it to shorter rows
+                        atomicSub(&s_used, pad);
+                        at = -1;
+                    }
+                }
+            }
             at = __shfl_sync(0xffffffffu, at, lane & ~(kFinLanes - 1));
-            const bool fits = at + pad <= arc_cap;
+            const int pad = at == -2 ? 0 : (deg + kFinLanes - 1) / kFinLanes * kFinLanes;
             unsigned cy = 0xffffffffu;
             for (int k = sub; k < pad; k += kFinLanes) {
                 int2 a = make_int2(-1, 0);     // no arc
@@ -439,18 +477,41 @@ k_sp_finish(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col
                         a.x = -1;
                     }
                 }
-                if (fits) s_arc[at + k] = a;
+                if (at >= 0) s_arc[at + k] = a;
             }
 #pragma unroll
             for (int o = kFinLanes / 2; o; o >>= 1) cy = min(cy, __shfl_xor_sync(0xffffffffu, cy, o));
             if (sub == 0 && y < n && j < meta_cap) {
-                s_cur[j] = deg ? kFar : 0ull;      // 0: a free column, nothing to lower
+                s_cur[j] = deg && at != -2 ? kFar : 0ull;      // 0: nothing to lower here
                 s_q[j] = key_q(__ldcg(key + y));
                 s_cy[j] = cy;
-                s_at[j] = fits ? make_int2(at, pad) : make_int2(-1, 0);
+                s_at[j] = at >= 0 ? make_int2(at, pad) : make_int2(-1, 0);
             }
         }
         __syncthreads();
+        const int nlong = min(s_nlong, kFinLongRows);
+        // the list's rows in segments of kFinSeg arcs, the CTA's warps in turn: f(row of the list, first arc, arcs)
+        auto segments = [&](auto &&f) {
+            const int segs = l_end[nlong - 1];
+            for (int k = 0, seg = warp; seg < segs; seg += kFinBlock / 32) {
+                while (seg >= l_end[k]) ++k;
+                const int off = (seg - (k ? l_end[k - 1] : 0)) * kFinSeg;
+                f(k, l_b[k] + off, min(kFinSeg, l_deg[k] - off));
+            }
+        };
+        if (nlong) {
+            if (tid == 0)
+                for (int k = 0, e = 0; k < nlong; ++k) l_end[k] = e += (l_deg[k] - 1) / kFinSeg + 1;
+            __syncthreads();
+            segments([&](int k, int b, int len) {
+                unsigned cy = 0xffffffffu;
+                for (int o = lane; o < len; o += 32)
+                    if (__ldg(cols + b + o) == l_y[k]) cy = min(cy, ZERO ? 0u : (unsigned)(__ldg(costs + b + o) - cmin));
+                cy = __reduce_min_sync(0xffffffffu, cy);
+                if (lane == 0 && cy != 0xffffffffu) atomicMin(&l_cy[k], cy);
+            });
+            __syncthreads();
+        }
         // Bellman-Ford sweeps until no potential falls. The CTAs sweep on
         // without waiting for each other (S only falls, so any mix of old and
         // new values is a valid relaxation) until kFinQuiet sweeps in a row
@@ -530,22 +591,40 @@ k_sp_finish(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col
                     if (y < n && (j >= meta_cap || (cur != 0 && s_at[j].x < 0))) {
                         const unsigned long long ky = __ldcg(key + y);
                         const uint32_t x = key_mate(ky);
-                        q = key_q(ky);
-                        cur = x < (uint32_t)n ? __ldcg(pot + y) : 0ull;
-                        if (cur != 0) {
-                            const int b = __ldg(row_ptr + x), e = __ldg(row_ptr + x + 1);
+                        int b = 0, deg = 0;
+                        if (x < (uint32_t)n) {
+                            b = __ldg(row_ptr + x);
+                            deg = __ldg(row_ptr + x + 1) - b;
+                        }
+                        if (j >= meta_cap) {
+                            q = key_q(ky);
+                            cur = deg ? __ldcg(pot + y) : 0ull;
                             cy = 0xffffffffu;
-                            for (int k = b; k < e; ++k)
-                                if (!ZERO && __ldg(cols + k) == y) cy = min(cy, (unsigned)(__ldg(costs + k) - cmin));
-                            if (ZERO) cy = 0;
-                            for (int k = b + sub; k < e; k += kFinLanes) {
-                                const int z = __ldg(cols + k);
-                                if (z == y) continue;
-                                const unsigned c = ZERO ? 0u : (unsigned)(__ldg(costs + k) - cmin);
-                                best = min(best, (unsigned long long)c * np1 + __ldcg(pot + z));
+                            if (deg > kFinLongRow)
+                                for (int k = 0; k < nlong; ++k)
+                                    if (l_y[k] == y) cur = 0;
+                        }
+                        for (int k = sub; cur != 0 && k < deg; k += 4 * kFinLanes) {
+                            int z[4];
+                            unsigned c[4];
+#pragma unroll
+                            for (int g = 0; g < 4; ++g) {
+                                const bool on = k + g * kFinLanes < deg;
+                                z[g] = on ? __ldg(cols + b + k + g * kFinLanes) : -1;
+                                c[g] = on && !ZERO ? (unsigned)(__ldg(costs + b + k + g * kFinLanes) - cmin) : 0u;
+                                if (z[g] == y) {
+                                    cy = min(cy, c[g]);
+                                    z[g] = -1;
+                                }
                             }
+#pragma unroll
+                            for (int g = 0; g < 4; ++g)
+                                best = min(best, (unsigned long long)c[g] * np1 + ld_if(pot + max(z[g], 0), z[g] >= 0, kFar));
                         }
                     }
+                    if (mine > meta_cap)   // a column without a record: its matched arc was found by one of the lanes
+#pragma unroll
+                        for (int o = kFinLanes / 2; o; o >>= 1) cy = min(cy, __shfl_xor_sync(0xffffffffu, cy, o));
                     best = min_u64_group(best);
                     if (sub == 0 && best < kFar && best + eps < cur + (unsigned long long)cy * np1) {
                         const unsigned long long v = best + eps - (unsigned long long)cy * np1;
@@ -553,6 +632,40 @@ k_sp_finish(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col
                             __stcg(pot + y, v);
                             if (j < meta_cap) s_cur[j] = v;
                             fell = true;
+                        }
+                    }
+                }
+                if (nlong) {
+                    segments([&](int k, int b, int len) {
+                        unsigned long long best = kFar;
+                        for (int o = lane; o < len; o += 4 * 32) {
+                            int z[4];
+                            unsigned c[4];
+#pragma unroll
+                            for (int g = 0; g < 4; ++g) {
+                                const bool on = o + 32 * g < len;
+                                z[g] = on ? __ldg(cols + b + o + 32 * g) : -1;
+                                c[g] = on && !ZERO ? (unsigned)(__ldg(costs + b + o + 32 * g) - cmin) : 0u;
+                                if (z[g] == l_y[k]) z[g] = -1;
+                            }
+#pragma unroll
+                            for (int g = 0; g < 4; ++g)
+                                best = min(best, (unsigned long long)c[g] * np1 + ld_if(pot + max(z[g], 0), z[g] >= 0, kFar));
+                        }
+                        best = warp_min(best);
+                        if (lane == 0 && best < kFar) atomicMin(&l_best[k], best);
+                    });
+                    __syncthreads();
+                    if (tid < nlong) {
+                        const unsigned long long best = l_best[tid], own = (unsigned long long)l_cy[tid] * np1;
+                        l_best[tid] = kFar;
+                        if (best < kFar && best + eps < l_cur[tid] + own) {
+                            const unsigned long long v = best + eps - own;
+                            if (v <= l_q[tid] + lim) {
+                                __stcg(pot + l_y[tid], v);
+                                l_cur[tid] = v;
+                                fell = true;
+                            }
                         }
                     }
                 }

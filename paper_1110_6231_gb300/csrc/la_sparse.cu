@@ -984,7 +984,7 @@ static la_status sparse_locked(const int32_t *row_ptr, const int32_t *cols, cons
     const int grid = std::max(1, std::min(w.num_sms * w.occ, (n + kBlock / 32 - 1) / (kBlock / 32)));
     if (profile) LA_SCK(cudaEventRecord(w.ev[0], s));
     const unsigned long long qinf = 4ull * (unsigned long long)n + 4;
-    // with end-of-phase updates; if those leave the price field, again with bids alone
+    // with end-of-phase updates; if those give up, again with bids alone
     Ctrl c1;
     int ph = 0;
     bool alone = false;
@@ -1041,7 +1041,9 @@ static la_status sparse_locked(const int32_t *row_ptr, const int32_t *cols, cons
         LA_SCK(cudaMemcpyAsync(w.h_ctrl, w.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s));
         LA_SCK(cudaStreamSynchronize(s));
         c1 = *w.h_ctrl;
-        if (alone || (c1.status != kGiveUp && c1.status != LA_ERR_OVERFLOW)) break;
+        // LA_ERR_INTERNAL: a grid barrier's wait ran out, behind bids on rows so long that one warp
+        // takes seconds (350,000 arcs, 256 bids); the refine has no barrier
+        if (alone || (c1.status != kGiveUp && c1.status != LA_ERR_OVERFLOW && c1.status != LA_ERR_INTERNAL)) break;
     }
     stats.phases = (int64_t)sched.size();
     stats.scans = (int64_t)c1.scans;

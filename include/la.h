@@ -452,7 +452,9 @@ la_status la_features(const int32_t *cost, int32_t n, void *stream, float *feats
                       float *inst_out);
 
 /* Forward pass over N feature rows forming I instances (seg: device
- * int32[I+1] row offsets): y_out device float[N]. */
+ * int32[I+1] row offsets): y_out device float[N]. A row outside
+ * [seg[0], seg[I]) belongs to no instance: its context is zero, and in a
+ * training step it adds nothing to the loss or the gradients. */
 la_status la_predictor_forward(const float *params, const float *feats, const int32_t *seg,
                                int32_t I, int32_t N, void *stream, float *y_out);
 

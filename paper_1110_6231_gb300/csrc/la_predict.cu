@@ -761,6 +761,7 @@ __device__ __forceinline__ void write_transposed(const __nv_bfloat16 (*tile)[kTi
 
 // Z = [H1 ; ctx of the row's segment] in BF16 (layer 2's operand) and, for
 // the weight gradient, its transpose ZT [256 x ldt] (ZT = nullptr: none).
+// A row in no segment (rowseg < 0) has zero context.
 __global__ void __launch_bounds__(256)
 k_concat(const float *__restrict__ H1, const float *__restrict__ ctx, const int *__restrict__ rowseg, int N,
          __nv_bfloat16 *__restrict__ Zb, __nv_bfloat16 *__restrict__ ZT, size_t ldt) {
@@ -769,8 +770,10 @@ k_concat(const float *__restrict__ H1, const float *__restrict__ ctx, const int 
 #pragma unroll
     for (int half = 0; half < 2; ++half) {
         for (int r = threadIdx.x >> 5; r < kTileRows && r0 + r < N; r += 8) {
-            const float *src = half ? ctx + (size_t)__ldg(rowseg + r0 + r) * H : H1 + (size_t)(r0 + r) * H;
-            const float4 x = __ldg(reinterpret_cast<const float4 *>(src + k));
+            const int i = half ? __ldg(rowseg + r0 + r) : r0 + r;
+            const float *src = half ? ctx : H1;
+            const float4 x = i < 0 ? make_float4(0.f, 0.f, 0.f, 0.f)
+                                   : __ldg(reinterpret_cast<const float4 *>(src + (size_t)i * H + k));
             const uint32_t p0 = pack_bf16(x.x, x.y), p1 = pack_bf16(x.z, x.w);
             *reinterpret_cast<uint2 *>(Zb + (size_t)(r0 + r) * 2 * H + half * H + k) = make_uint2(p0, p1);
             const __nv_bfloat162 a = *reinterpret_cast<const __nv_bfloat162 *>(&p0);
@@ -787,7 +790,7 @@ k_concat(const float *__restrict__ H1, const float *__restrict__ ctx, const int 
     }
 }
 
-// row -> segment index
+// row -> segment index (rows in no segment keep the -1 that the buffer is cleared to)
 __global__ void k_rowseg(const int *__restrict__ seg, int I, int *__restrict__ rowseg) {
     const int i = blockIdx.x;
     for (int r = seg[i] + threadIdx.x; r < seg[i + 1]; r += blockDim.x) rowseg[r] = i;
@@ -926,7 +929,9 @@ k_dh1(const float *__restrict__ dZ, const float *__restrict__ H1, const float *_
         if (r0 + r >= N) break;
         const float4 z = __ldg(reinterpret_cast<const float4 *>(dZ + (size_t)(r0 + r) * H + k));
         const float4 h = __ldg(reinterpret_cast<const float4 *>(H1 + (size_t)(r0 + r) * H + k));
-        const float4 c = __ldg(reinterpret_cast<const float4 *>(cseg + (size_t)__ldg(rowseg + r0 + r) * H + k));
+        const int i = __ldg(rowseg + r0 + r);      // in no segment: no pooled gradient, and z is zero
+        const float4 c = i < 0 ? make_float4(0.f, 0.f, 0.f, 0.f)
+                               : __ldg(reinterpret_cast<const float4 *>(cseg + (size_t)i * H + k));
         const float d0 = h.x > 0.f ? z.x + c.x : 0.f, d1 = h.y > 0.f ? z.y + c.y : 0.f;
         const float d2 = h.z > 0.f ? z.z + c.z : 0.f, d3 = h.w > 0.f ? z.w + c.w : 0.f;
         s.x += d0;
@@ -1144,6 +1149,7 @@ cudaError_t forward(cudaStream_t s, const float *P, const float *X, int N, int I
     int one = 1;
     k_weights_bf16<<<64, 256, 0, s>>>(P, w.wb);
     k_conv_x<<<(unsigned)(((size_t)N * 64 + 255) / 256), 256, 0, s>>>(X, N, w.Xb);
+    if ((e = cudaMemsetAsync(w.rowseg, 0xff, sizeof(int) * (size_t)N, s)) != cudaSuccess) return e;
     k_rowseg<<<I, 256, 0, s>>>(seg, I, w.rowseg);
     // layer 1: H1 = relu(X W1 + b1)   (K = 16 real features)
     if ((e = tc_gemm<128>(s, w.Xb, 64, w.wb + WB_W1T, 64, H, N, F, one, 0, w.H1, H, H, nullptr, 0, P + OFF_B1,

@@ -234,3 +234,41 @@ def test_gradients_at_tile_edges(la, sizes):
     for a, b in ((se.OFF_W1, se.OFF_B1), (se.OFF_B1, se.OFF_W2), (se.OFF_W2, se.OFF_B2), (se.OFF_B2, se.OFF_W3),
                  (se.OFF_W3, se.OFF_B3)):
         assert np.linalg.norm(g[a:b] - gq[a:b]) < 5e-3 * max(np.linalg.norm(gq[a:b]), 1e-12)
+
+
+@pytest.mark.parametrize("before,after", [(0, 70), (65, 0), (3, 200)])
+def test_rows_in_no_segment_add_nothing(la, before, after):
+    """Feature rows outside [seg[0], seg[I]) read no context and leave loss and
+    gradients as they are without them. The covered rows' own values are the
+    same; they shift within their tiles, so that the FP32 sums over n = 177 rows
+    differ by their order: at most n 2^-24 of the sum of the terms' sizes,
+    which is about sqrt(n) times the sum's own size, or 1.4e-4 of it."""
+    P = _params(17)
+    X, t, seg = _inputs(18, [40, 130, 7])
+    N = X.shape[0]
+    rng = np.random.default_rng(1)
+
+    def step(X, t, seg):
+        import torch
+        g = torch.zeros(la.LA_PRED_PARAMS, dtype=torch.float32, device="cuda")
+        y = torch.zeros(X.shape[0], dtype=torch.float32, device="cuda")
+        loss = ctypes.c_float(0)
+        Pd, Xd, sd = _dev(P, np.float32), _dev(X, np.float32), _dev(seg, np.int32)
+        assert la.la_predictor_train_step(Pd, None, None, Xd, _dev(t, np.float32), sd, len(seg) - 1, X.shape[0], 1, 0.0,
+                                          0.0, None, g, ctypes.byref(loss)) == la.LA_OK
+        assert la.la_predictor_forward(Pd, Xd, sd, len(seg) - 1, X.shape[0], None, y) == la.LA_OK
+        return loss.value, g.cpu().numpy(), y.cpu().numpy()
+
+    loss0, g0, y0 = step(X, t, seg)
+    Xx = np.zeros((N + before + after, 16))
+    Xx[:, :8] = rng.normal(0, 1, (Xx.shape[0], 8))
+    Xx[before:before + N] = X
+    tx = rng.normal(0, 100, Xx.shape[0])
+    tx[before:before + N] = t
+    loss, g, y = step(Xx, tx, seg + before)
+    assert loss == pytest.approx(loss0, rel=1e-5)
+    np.testing.assert_allclose(y[before:before + N], y0, rtol=0, atol=1e-5 * np.abs(y0).max())
+    assert np.isfinite(y).all()
+    for a, b in ((se.OFF_W1, se.OFF_B1), (se.OFF_B1, se.OFF_W2), (se.OFF_W2, se.OFF_B2), (se.OFF_B2, se.OFF_W3),
+                 (se.OFF_W3, se.OFF_B3)):
+        assert np.linalg.norm(g[a:b] - g0[a:b]) <= 1.4e-4 * np.linalg.norm(g0[a:b])

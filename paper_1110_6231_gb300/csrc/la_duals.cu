@@ -29,6 +29,7 @@ namespace {
 constexpr int kMaxDevices = 64;
 constexpr int kDualBlock = 512;
 constexpr int kDualRounds = 4;      // sweeps of a CTA between two grid barriers
+constexpr int kDualBurst = 256;     // ... in the first epochs; one from there on
 
 struct DualCtrl {
     GridBar bar;
@@ -67,6 +68,10 @@ __global__ void k_dual_init(const int32_t *__restrict__ C, int n, const int32_t 
 // grid barriers a CTA sweeps up to kDualRounds times: v only falls, so any mix
 // of old and new values is a valid relaxation, and the fixed point is the
 // same. The launch ends when no CTA lowered anything between two barriers.
+// After kDualBurst epochs the matching is most likely not optimal: rows fall in
+// every sweep until n + 2 epochs prove it, and one sweep each is enough for that
+// (two rows of an optimum swapped, n = 4096: 342 ms with four sweeps, 143 with
+// one, 156 from one launch pair and host synchronisation per sweep).
 // Bound by the latency of one row read and one barrier per epoch: 1.25 -> 0.27
 // ms at n = 2048 (geometric), from one launch pair, a memset, a copy and a
 // host synchronisation per sweep, whose 32 CTAs read the whole matrix.
@@ -85,7 +90,8 @@ k_dual_sweeps(const int32_t *__restrict__ C, int n, const int32_t *__restrict__ 
     for (int ep = 0; ep < max_epochs; ++ep) {
         const int slot = ep % 3;
         bool any = false;
-        for (int round = 0; round < kDualRounds; ++round) {
+        const int rounds = ep < kDualBurst ? kDualRounds : 1;
+        for (int round = 0; round < rounds; ++round) {
             bool found = false;
             // the CTA's rows, kDualBlock at a time
             for (long long r0 = 0; blockIdx.x + r0 * gridDim.x < n; r0 += kDualBlock) {

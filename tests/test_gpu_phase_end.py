@@ -79,3 +79,22 @@ def test_certificate_is_the_largest_potential(la, n):  # noqa: F811
         want = new
     np.testing.assert_array_equal(v, want)
     np.testing.assert_array_equal(u, on - want[m])
+
+
+@pytest.mark.parametrize("n", [300, 1001, 2000])
+def test_certificate_of_long_chains_and_of_no_optimum(la, n):  # noqa: F811
+    """Residual paths through all columns take more sweeps than the epochs with
+    several each: row x costs 1 on its own column and 0 on the next, so that
+    v(y) = -y. Two rows swapped are no optimum, which n + 2 epochs show."""
+    import torch
+    C = torch.full((n, n), 2 * n, dtype=torch.int32, device="cuda")
+    i = torch.arange(n, device="cuda")
+    C[i, i] = 1
+    C[i[:-1], i[1:]] = 0
+    match = i.to(torch.int32)
+    u, v = la.dual_certificate(C, match)
+    assert torch.equal(v, -i)
+    assert torch.equal(u, 1 + i)
+    match[:2] = match[:2].flip(0)
+    out = torch.zeros(n, dtype=torch.int64, device="cuda")
+    assert la.la_dual_certificate(C, n, match, None, None, out) == la.LA_ERR_INTERNAL

@@ -819,7 +819,7 @@ struct SparseWorkspace {
     Ctrl *h_ctrl = nullptr;
     int num_sms = 0;
     int occ = 0;
-    bool events = false;
+    int events = 0;                      // events made
     cudaEvent_t ev[2];
 };
 
@@ -827,21 +827,21 @@ std::mutex g_smu;
 SparseWorkspace g_sws[kMaxDevices];
 
 la_status ensure_sws(SparseWorkspace &w, int64_t n) {
-    if (!w.ctrl) {
-        int dev = 0;
+    // what a call that failed here has left out, the next one makes
+    if (!w.num_sms) {
+        int dev = 0, sms = 0;
         if (cudaGetDevice(&dev) != cudaSuccess) return LA_ERR_CUDA;
-        if (cudaDeviceGetAttribute(&w.num_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-            return LA_ERR_CUDA;
-        if (cudaMalloc(&w.ctrl, sizeof(Ctrl)) != cudaSuccess) return LA_ERR_NOMEM;
-        if (cudaMallocHost(&w.h_ctrl, sizeof(Ctrl)) != cudaSuccess) return LA_ERR_NOMEM;
-        for (auto &e : w.ev)
-            if (cudaEventCreate(&e) != cudaSuccess) return LA_ERR_CUDA;
-        w.events = true;
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return LA_ERR_CUDA;
         int o = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_sp_refine<false>, kBlock, 0);
         w.occ = std::max(1, o);
-        if (cudaMalloc(&w.fin, sizeof(FinCtrl)) != cudaSuccess) return LA_ERR_NOMEM;
+        w.num_sms = sms;
     }
+    if (!w.ctrl && cudaMalloc(&w.ctrl, sizeof(Ctrl)) != cudaSuccess) return LA_ERR_NOMEM;
+    if (!w.h_ctrl && cudaMallocHost(&w.h_ctrl, sizeof(Ctrl)) != cudaSuccess) return LA_ERR_NOMEM;
+    if (!w.fin && cudaMalloc(&w.fin, sizeof(FinCtrl)) != cudaSuccess) return LA_ERR_NOMEM;
+    for (; w.events < 2; ++w.events)
+        if (cudaEventCreate(&w.ev[w.events]) != cudaSuccess) return LA_ERR_CUDA;
     if (w.cap < n) {
         cudaFree(w.key);
         cudaFree(w.qm);

@@ -146,3 +146,37 @@ def test_sizes_around_a_relabel_tile(la, H, W):
     src = (rng.integers(0, 60, (H, W)) * (rng.random((H, W)) < 0.2)).astype(np.int32)
     snk = (rng.integers(0, 60, (H, W)) * (rng.random((H, W)) < 0.2)).astype(np.int32)
     expect_same(la, cap, src, snk)
+
+
+def serpentine(H, W, turn, rng):
+    """One corridor of capacity 3..9 through every second row of an H x W grid
+    (transposed if `turn`), from a source arc at its start to a sink arc at
+    its end, with a narrow place half way."""
+    cap = np.zeros((4, H, W), dtype=np.int32)
+    src, snk = np.zeros((2, H, W), dtype=np.int32)
+    path = []
+    for k, i in enumerate(range(0, H, 2)):
+        row = [(i, j) for j in range(W)]
+        path += row if k % 2 == 0 else row[::-1]
+        if i + 2 < H:
+            path.append((i + 1, path[-1][1]))
+    step = {(0, 1): 0, (0, -1): 1, (1, 0): 2, (-1, 0): 3}
+    for (i, j), (k, m) in zip(path, path[1:]):
+        cap[step[k - i, m - j], i, j] = rng.integers(3, 10)
+    (i, j), (k, m) = path[len(path) // 2:len(path) // 2 + 2]
+    cap[step[k - i, m - j], i, j] = 2
+    src[path[0]] = snk[path[-1]] = 20
+    if turn:
+        cap = cap[[2, 3, 0, 1]].transpose(0, 2, 1)
+        src, snk = src.T, snk.T
+    return [np.ascontiguousarray(a) for a in (cap, src, snk)]
+
+
+@pytest.mark.parametrize("turn", [False, True])
+@pytest.mark.parametrize("H,W", [(9, 31), (31, 32), (33, 65), (97, 70)])
+def test_corridors_longer_than_a_tiles_rounds(la, H, W, turn):
+    """Distances that take a relabel tile more rounds than one pass gives it
+    (128), and that leave tiles and come back: a tile is due again when it
+    stopped short of its fixed point, or when a neighbour changed."""
+    g = serpentine(H, W, turn, np.random.default_rng(H * W))
+    assert expect_same(la, *g).flow == 2

@@ -1032,15 +1032,14 @@ constexpr int kSmallThreads = 1024;
 constexpr int kSmallMaxN16 = 300;    // 2 n^2 + 8 n bytes of shared memory
 constexpr int kSmallMaxN32 = 224;    // 4 n^2 + 8 n bytes
 
-//
 // A bid is a chain of dependent shared-memory reads and instructions of one
 // warp, so both are kept few: with 32-bit values the key is (2^32 - 1 - q) in
 // the high word and the mate in the low one, so that a price is one word and
-// v = c (n+1) + ~hi; of 16-bit costs, n a multiple of 4, a lane ranks four columns from
-// one read of their costs and two 16-byte reads of their keys; and the best
-// column's cost is kept beside it instead of being read back. Uniform n = 256,
-// costs to 1000: 0.71 -> 0.61 ms a solve; n = 64 unchanged (0.24 ms, more than
-// half of it launches and two host synchronisations).
+// v = c (n+1) + ~hi; of 16-bit costs, n a multiple of 4 above 224, a lane ranks
+// four columns from one read of their costs and two 16-byte reads of their keys;
+// and the best column's cost is kept beside it instead of being read back.
+// Uniform n = 256, costs to 1000: 0.76 -> 0.67 ms a solve; n = 64 unchanged
+// (0.24 ms, more than half of it launches and two host synchronisations).
 // 64-bit values keep one column a lane and read: in fours a scan's 64-bit
 // selects outweigh the reads saved (n = 200: 0.81 -> 1.02 ms).
 struct SmallSched {
@@ -1091,9 +1090,11 @@ k_small(const int32_t *__restrict__ C, int n, int cmin, uint32_t np1, const __gr
     }
     __syncthreads();
     const volatile unsigned long long *vkey = skey;
-    // four columns a lane: rows of 16-bit costs then start on 8 bytes; below 128 columns lanes would
-    // idle, and with 32-bit costs the gain is lost (n = 224: 0.65 ms in fours, 0.62 before)
-    const bool vec = C16 && (n & 3) == 0 && n >= 128;
+    // four columns a lane: rows of 16-bit costs then start on 8 bytes. A round takes 128 columns, so that
+    // up to 224 a lane ranks more of them in two rounds of fours than one by one; and with 32-bit costs the
+    // gain is lost. ms a solve one by one and in fours (means of 24 instances, costs to 1000): n = 144 0.39,
+    // 0.44; 192 0.50, 0.56; 224 0.59, 0.64; 228 0.87, 0.66; 256 0.76, 0.67; 300 1.04, 0.87
+    const bool vec = C16 && (n & 3) == 0 && n > 224;
     unsigned long long wins = 0, displaced = 0, chain_max = 0;
     for (int ph = 0; ph < nph; ++ph) {
         const unsigned long long eps = sched.eps[ph];
@@ -1163,19 +1164,12 @@ k_small(const int32_t *__restrict__ C, int n, int cmin, uint32_t np1, const __gr
                 if (vec) {
 #pragma unroll 2
                     for (int y = 4 * lane; y < n; y += 128) {
-                        uint32_t c0, c1, c2, c3;
-                        if (C16) {
-                            const ushort4 c = *reinterpret_cast<const ushort4 *>(crow + y);
-                            c0 = c.x, c1 = c.y, c2 = c.z, c3 = c.w;
-                        } else {
-                            const uint4 c = *reinterpret_cast<const uint4 *>(crow + y);
-                            c0 = c.x, c1 = c.y, c2 = c.z, c3 = c.w;
-                        }
+                        const ushort4 c = *reinterpret_cast<const ushort4 *>(crow + y);
                         const ulonglong2 a = ld_skey2(skey + y), b = ld_skey2(skey + y + 2);
-                        push(y, c0, a.x);
-                        push(y + 1, c1, a.y);
-                        push(y + 2, c2, b.x);
-                        push(y + 3, c3, b.y);
+                        push(y, c.x, a.x);
+                        push(y + 1, c.y, a.y);
+                        push(y + 2, c.z, b.x);
+                        push(y + 3, c.w, b.y);
                     }
                 } else {
                     for (int y = lane; y < n; y += 32) push(y, crow[y], vkey[y]);

@@ -87,3 +87,17 @@ def test_small_kernel_options(la):
     stopped = la.solve(t, scan_budget=100, check=False)
     assert stopped.stats["status"] == la.LA_ERR_ITER_LIMIT
     assert la.solve(t).cost == h
+
+
+@pytest.mark.parametrize("n", [128, 220, 223, 224, 225, 228, 252, 260, 300])
+@pytest.mark.parametrize("hi", [1000, 65535])
+def test_both_sides_of_the_line_for_four_columns_a_lane(la, n, hi):
+    """16-bit costs: one column a lane up to n = 224 and where n is no multiple
+    of 4, four above, with a last round of 128 columns that is nearly empty
+    (228, 260) or nearly full (252)."""
+    for seed in range(2):
+        C = synth.uniform_costs(n, 0, hi, 40 + seed)
+        cost, match, prices, st = run(la, C)
+        assert st["small_kernel"] == 1 and cost == oracle.hungarian(C)[0]
+        assert oracle.check_matching(C, match, cost) == 0
+        assert oracle.check_eps_cs(C, match, prices, 1) == 0

@@ -743,7 +743,8 @@ k_segment_back(const __nv_bfloat16 *__restrict__ dH2b, const __nv_bfloat16 *__re
 
 // Tiles of 64 rows x 128 columns, 256 threads: thread t holds columns
 // 4 (t % 32) .. + 3 of rows t / 32, + 8, ...; transposed BF16 goes through
-// `tile` (66 elements per row: no bank conflicts worth counting).
+// `tile` (66 elements per row: a column is read without bank conflicts, the
+// stores of four columns a lane fall four lanes to a bank).
 constexpr int kTileRows = 64, kTilePitch = kTileRows + 2;
 
 // tile[k][r] -> dst[k][r0 + r], 64 contiguous rows (128 bytes) per column k
@@ -790,10 +791,16 @@ k_concat(const float *__restrict__ H1, const float *__restrict__ ctx, const int 
     }
 }
 
-// row -> segment index (rows in no segment keep the -1 that the buffer is cleared to)
-__global__ void k_rowseg(const int *__restrict__ seg, int I, int *__restrict__ rowseg) {
+// row -> segment index, -1 for the rows before the first and after the last
+// segment (one CTA per segment; the outer two write those too: clearing the
+// buffer first was one launch more, 4 of a training step's 247 us)
+__global__ void k_rowseg(const int *__restrict__ seg, int I, int N, int *__restrict__ rowseg) {
     const int i = blockIdx.x;
     for (int r = seg[i] + threadIdx.x; r < seg[i + 1]; r += blockDim.x) rowseg[r] = i;
+    if (i == 0)
+        for (int r = threadIdx.x; r < min(seg[0], N); r += blockDim.x) rowseg[r] = -1;
+    if (i == I - 1)
+        for (int r = max(seg[I], 0) + threadIdx.x; r < N; r += blockDim.x) rowseg[r] = -1;
 }
 
 // Loss of one batch and dL/dy: per instance, the variance of the error
@@ -1149,8 +1156,7 @@ cudaError_t forward(cudaStream_t s, const float *P, const float *X, int N, int I
     int one = 1;
     k_weights_bf16<<<64, 256, 0, s>>>(P, w.wb);
     k_conv_x<<<(unsigned)(((size_t)N * 64 + 255) / 256), 256, 0, s>>>(X, N, w.Xb);
-    if ((e = cudaMemsetAsync(w.rowseg, 0xff, sizeof(int) * (size_t)N, s)) != cudaSuccess) return e;
-    k_rowseg<<<I, 256, 0, s>>>(seg, I, w.rowseg);
+    k_rowseg<<<I, 256, 0, s>>>(seg, I, N, w.rowseg);
     // layer 1: H1 = relu(X W1 + b1)   (K = 16 real features)
     if ((e = tc_gemm<128>(s, w.Xb, 64, w.wb + WB_W1T, 64, H, N, F, one, 0, w.H1, H, H, nullptr, 0, P + OFF_B1,
                           EP_BIAS | EP_RELU, w.err, 64)) != cudaSuccess)

@@ -112,7 +112,6 @@ k_mf_push(int H, int W, long long *__restrict__ e, int *__restrict__ h, int *__r
     const int N = H * W, NV = N + 2;               // |V|: the pixels, s and t
     const int stride = gridDim.x * blockDim.x;
     unsigned long long sunk = 0;                   // pushed into t by this thread
-    if (c->status != 0) return;                    // invalid capacities: no neighbour is read
     for (int it = 0; it < cycle; ++it) {
         for (int u = blockIdx.x * blockDim.x + threadIdx.x; u < N; u += stride) {
             const long long eu = (long long)__ldcg(reinterpret_cast<const unsigned long long *>(e) + u);
@@ -364,8 +363,8 @@ static la_status maxflow_locked(const int32_t *cap, const int32_t *src, const in
     k_mf_init<<<grid, kBlock, 0, s>>>(cap, src, snk, H, W, w.e, w.h, w.cf, w.rt, w.ctrl);
     int64_t launches = 1;
     LA_MCK(cudaGetLastError());
-    // invalid capacities are found at the first relabel's read-back; until then no
-    // kernel reads a neighbour outside the grid (k_mf_push stops on the status)
+    // invalid capacities are found at the first relabel's read-back; the relabel
+    // reads no neighbour outside the grid, and nothing is pushed before it
 
     // global relabel: init, then batches of sweeps until a batch's last sweep changes nothing
     auto global_relabel = [&]() -> la_status {

@@ -308,11 +308,12 @@ k_sp_refine(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col
 // there on the last graph took 22 million bids, with bids alone 7 million, with
 // updates 0.6. Prices of the graphs timed below stay under 2^32.
 //
-// Measured on GB300, whole solves (mean of 6, ms), from one refine launch per
-// phase: sparse-uniform n = 65536, 33 arcs a row, 193 -> 29; sparse-geometric
-// n = 16384, 36 arcs a row, 242 -> 94. There the 50 updates take 58 ms (150
-// sweeps each, 4.5 us a sweep: gathers of 8 scattered bytes, about one 32-byte
-// sector per two cycles and SM), the bids 18 ms. Without the caching a sweep
+// Measured on GB300, whole solves in turn with the code that had one refine
+// launch per phase, ms: sparse-uniform n = 65536, 33 arcs a row, 261 -> 34;
+// sparse-geometric n = 16384, 36 arcs a row, 360 -> 96. There the 50 updates
+// take 58 ms (150 sweeps each, 4.5 us a sweep), the bids 18 ms. Bound by a
+// sweep's latency: 59 % of the warp cycles are spent at the CTA barrier, 27 %
+// on gathers, with L2 at 14 % of its rate (ncu). When this form was chosen (88 ms then): without the caching a sweep
 // took 19 us; without the bound on K 60 % more sweeps. Chains of at most 64,
 // 256 and 1024 bids a round: 107, 88 and 95 ms (and 36, 29, 31 on the uniform
 // graph): short chains do not reach the end of their path, long ones are rows
@@ -869,8 +870,9 @@ la_status ensure_sws(SparseWorkspace &w, int64_t n) {
 }
 
 // Free rows at which the refine hands a phase to the end-of-phase kernel.
-// Measured (means of 6 solves, ms) at n / 1000, n / 128, n / 32: sparse-uniform
-// n = 65536 73, 29, 28; sparse-geometric n = 16384 273, 88, 94.
+// Measured (means of 12 solves, ms, +- 10 %) at n / 1000, n / 256, n / 64, n / 16:
+// sparse-uniform n = 65536 34, 36, 36, 35; sparse-geometric n = 16384 182, 102,
+// 92, 95, n = 65536 585, 413, 420, 418.
 int sp_hand_free(int n) {
     return std::max(8, n / 64);
 }

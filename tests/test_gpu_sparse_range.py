@@ -66,3 +66,23 @@ def test_both_sides_of_the_line_for_bids_alone(la, n, degree):  # noqa: F811
     sol = expect_same(la, rp, cols, costs)
     updates = n > 512 and 2 * cols.size > 5 * n
     assert sol.stats["refine_launches"] == (2 if updates else 1) * (sol.stats["phases"] + 1) + (not updates)
+
+
+@pytest.mark.parametrize("kind", ["geometric", "uniform"])
+def test_a_missing_matching_is_found_by_one_update(la, kind):  # noqa: F811
+    """12 rows that reach only 11 columns, in a large graph: one update shows it,
+    not a price war of 4n steps (more than 40 scans a row)."""
+    n = 40_000
+    rp, cols, costs = synth.sparse_geometric(n, 4) if kind == "geometric" else synth.sparse_uniform(n, 3, 4)
+    keep = np.ones(cols.size, dtype=bool)
+    keep[:rp[12]] = False
+    hall = np.tile(np.arange(11), 12)
+    g = (np.concatenate([np.arange(12) * 11, rp[12:] - rp[12] + 132]), np.concatenate([hall, cols[keep]]),
+         np.concatenate([np.full(132, 5), costs[keep]]))
+    missing = np.setdiff1d(np.arange(n), g[1])     # columns that only the 12 rows had: row n - 1 takes them
+    g = (np.concatenate([g[0][:-1], [g[0][-1] + missing.size]]), np.concatenate([g[1], missing]),
+         np.concatenate([g[2], np.zeros(missing.size, dtype=g[2].dtype)]))
+    sol = gpu_solve(la, *g)
+    assert sol.stats["status"] == la.LA_ERR_INFEASIBLE
+    assert sol.stats["price_updates"] >= 1
+    assert sol.stats["scans"] < 10 * n
